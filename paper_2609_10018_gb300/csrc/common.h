@@ -91,6 +91,9 @@ enum GemmEpi : int {
   EPI_BIAS_RELU_F16 = ELASTO_EPI_BIAS_RELU_F16,
   EPI_BIAS_F16 = ELASTO_EPI_BIAS_F16,
   EPI_BIAS_RESID_RELU_F16 = ELASTO_EPI_BIAS_RESID_RELU_F16,
+  // EPI_BIAS_RESID_F32 whose residual is the output itself: the tile leaves by
+  // TMA reduce-add stores (gemm_plan picks it; gemm_set_residual_source undoes it)
+  EPI_BIAS_ADD_F32 = 100,
 };
 
 struct GemmArgs {
@@ -102,7 +105,7 @@ struct GemmArgs {
   int* status;
   int stages;             // operand ring depth (<= 8)
   int b_stage;            // bytes of one B stage (both planes; half of B for a CTA pair)
-  int cbufs;              // output staging buffers (16 KB each) for the TMA-store epilogues
+  int cbufs;              // output staging pieces (4 KB) of each epilogue warp, for the TMA-store epilogues
   int b_planes;           // 2: W held as bf16 hi + lo planes (fp32-stored models), both multiplied
   int pair;               // 1: clusters of two CTAs sharing 256-row tiles (tcgen05 cta_group::2)
   int f16;                // 1: A, W, the residual and 16-bit outputs are f16 (the *_F16 epilogues), else bf16
@@ -129,7 +132,7 @@ struct GemmArgs {
 
 struct GemmPlan {
   CUtensorMap tmA, tmB, tmB2;  // tmB2: low bf16 plane of W (b_planes == 2)
-  CUtensorMap tmC;        // output [M_cap, ldo] (bf16 or fp32), box 128 B x 128 rows, 128B swizzle
+  CUtensorMap tmC;        // output [M_cap, ldo] (bf16 or fp32), box 128 B x 32 rows, 128B swizzle
   CUtensorMap tmR;        // residual source of EPI_BIAS_RESID_F32 (the output itself by default)
   GemmArgs args;          // M here is the capacity the A map was encoded for
   int epi = 0;
@@ -147,8 +150,6 @@ struct GemmPlan {
   int ln_d = 0;
 };
 
-// Pick the N tile for an M x N problem.
-int gemm_pick_bn(int M, int N, int step = 32, bool pair = false);
 // Build maps/arguments for out = epi(A[M_cap, K] W[N, K]^T). A and W must stay
 // allocated for the plan's life.
 // W_lo (optional): second bf16 plane so that W = W + W_lo carries ~16

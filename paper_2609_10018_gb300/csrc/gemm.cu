@@ -15,20 +15,29 @@
 //    instead be loaded once per CTA and kept (b_resident: one N tile);
 //  - warp 1 lane 0: issues tcgen05.mma (M=128, N=bn, K=16) into one of two
 //    TMEM accumulators (2 x 256 fp32 columns), commits stages back to the
-//    producer and finished accumulators to the epilogue. K >= 1536 on
-//    256-row tiles: CTA pairs (cta_group::2, M = 256, each CTA holds half of
-//    B);
-//  - warps 2-17: epilogue, four warps per 32-lane quarter of TMEM (= 32 rows
-//    of the tile), each taking a quarter of every 64-column chunk.
-//    * bf16 outputs (QKV, FC1+GELU, conv+ReLU) and the fp32 residual stream
-//      (out-proj, FC2): each thread writes its row piece of a 128-row x
-//      128-byte chunk into a 128B-swizzled staging buffer in shared memory
-//      (bank conflict free 16-byte stores) and one thread stores the chunk
-//      with a TMA tensor store. For the residual, the old rows of X are
-//      brought into the same staging buffer by TMA loads issued several
-//      chunks ahead, so the read-modify-write of X runs at full memory
-//      parallelism. The 16-bit residual + ReLU of the CNN block outputs works
-//      the same way.
+//    producer and finished accumulators to the epilogue.
+//  - CTA pairs (cta_group::2, M = 256, each CTA holds half of B) where
+//    tile_cost() puts them ahead, at every K. What bounds a single 128 x 256
+//    tile is shared memory: per k-block the MMAs read 48 KB and TMA writes
+//    48 KB, 0.38 us at 128 B a clock, more than the 0.27 us the MMAs take, and
+//    the epilogue's staging comes on top. A pair's CTA reads 32 KB and writes
+//    32 KB. ViT-B QKV at batch 256 (50432 x 2304 x 768): 124 us single, 108 us
+//    pairs; FC1 + GELU 172 -> 157 us; 50432 x 3072 x 768 without GELU 160 ->
+//    141 us (a library bf16 GEMM of that size: 140 us).
+//  - warps 2-13: epilogue, three warps per 32-lane quarter of TMEM (= 32 rows
+//    of the tile). A warp works alone: it takes every third 128-byte-wide
+//    chunk of its rows from TMEM to registers, writes it to its own 4 KB
+//    staging piece (128B-swizzled, bank conflict free) and stores it with its
+//    own TMA box. 16 warps on quarter chunks behind a 512-thread barrier per
+//    chunk needed 4.9 us a tile, longer than a pair's main loop (3.7 us), most
+//    of it in the barrier and in bias loads from the loaded L2 path; eight
+//    warps on their own lack the overlap for GELU (FC1 174 us), sixteen the
+//    registers. GELU, bias and residual use packed fp32 pairs.
+//    * the fp32 residual stream (out-proj, FC2) leaves by TMA reduce-add: X is
+//      not read into the SM. FC2 (K = 3072) 158 -> 149 us, out-proj 76 -> 72.
+//      A plan of few tiles (or with another residual source) reads the old rows
+//      into the staging pieces ahead instead, as the 16-bit residual + ReLU of
+//      the CNN block outputs does.
 //    * the remaining epilogue (fp32 out) transposes through padded shared
 //      memory for row-contiguous stores (warps 2-5); it also writes the
 //      partial sums of a split-K plan, whose k-block range is
@@ -48,17 +57,21 @@ namespace elasto {
 namespace {
 
 constexpr int BM = 128, BK = 64, MAX_STAGES = 8, MAX_BN = 256;
-constexpr int EPI_THREADS = 512;                 // 16 epilogue warps, four per TMEM lane quarter
-constexpr int THREADS = 64 + EPI_THREADS;
-constexpr int THREADS_CONV = THREADS + 32;  // implicit convolutions: warp 18 is a second TMA producer
+constexpr int EPI_WARPS = 12;               // three epilogue warps per TMEM lane quarter
+constexpr int GROUPS = EPI_WARPS / 4;       // a group is one warp of every quarter: 128 rows
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
+constexpr int THREADS_CONV = THREADS + 32;  // implicit convolutions: warp 14 is a second TMA producer
 constexpr int A_STAGE = BM * BK * 2;        // 16 KB
-constexpr int CBUF = BM * 128;              // 16 KB staging chunk (128 rows x 128 B)
-constexpr int POOL = 224 * 1024;            // operand ring + staging buffers
-constexpr int MAX_CBUFS = 8;
+constexpr int WBUF = 32 * 128;              // 4 KB staging piece of one epilogue warp (32 rows x 128 B)
+constexpr int CBUF = EPI_WARPS * WBUF;      // 48 KB: one staging piece for every epilogue warp
+constexpr int POOL = 224 * 1024;            // operand ring + staging pieces
+constexpr int MAX_CBUFS = 2;                // staging pieces per epilogue warp
 constexpr int EPI_LD = 33;                  // padded row of the transpose tile
 constexpr int EPI_TILE = 32 * EPI_LD;       // floats per epilogue warp
 constexpr int TMEM_COLS = 512;
-constexpr size_t SMEM_BYTES = 1024 + POOL + 512;
+constexpr size_t SMEM_BYTES = 1024 + POOL + 2048;
+static_assert((2 * MAX_STAGES + 6 + EPI_WARPS * MAX_CBUFS) * 8 + 32 * EPI_WARPS * 4 + 4 * (1 + GROUPS) <= 2048,
+              "barriers and bias");
 
 template <int EPI>
 struct EpiTraits {
@@ -67,9 +80,11 @@ struct EpiTraits {
   // brought into the staging buffer by TMA like the fp32 residual stream
   static constexpr bool resid16 = EPI == EPI_BIAS_RESID_RELU_BF16 || EPI == EPI_BIAS_RESID_RELU_F16;
   static constexpr bool tma = EPI == EPI_BIAS_BF16 || EPI == EPI_BIAS_GELU_BF16 || EPI == EPI_BIAS_RELU_BF16 ||
-                              EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_RELU_F16 || EPI == EPI_BIAS_F16 ||
-                              resid16;
-  static constexpr bool f32 = EPI == EPI_BIAS_RESID_F32;
+                              EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32 || EPI == EPI_BIAS_RELU_F16 ||
+                              EPI == EPI_BIAS_F16 || resid16;
+  static constexpr bool f32 = EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32;
+  // the old value is read into the staging piece by TMA; EPI_BIAS_ADD_F32
+  // reads nothing: the store itself adds to memory
   static constexpr bool resid = EPI == EPI_BIAS_RESID_F32 || resid16;
   static constexpr int cw = f32 ? 32 : 64;  // columns per 128-byte staging chunk
 };
@@ -88,10 +103,10 @@ __device__ __forceinline__ int resid_row(const GemmArgs& a, int m0) {
 }
 
 template <int EPI>
-__device__ __forceinline__ float epi_act(float v) {
-  if constexpr (EPI == EPI_BIAS_GELU_BF16) return gelu(v);
+__device__ __forceinline__ float2 epi_act2(float2 v) {
+  if constexpr (EPI == EPI_BIAS_GELU_BF16) return gelu2(v);
   if constexpr (EPI == EPI_BIAS_RELU_BF16 || EPI == EPI_BIAS_RELU_F16 || EpiTraits<EPI>::resid16)
-    return fmaxf(v, 0.0f);
+    return make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f));
   return v;
 }
 
@@ -113,25 +128,6 @@ __device__ __forceinline__ uint32_t pack_out(float lo, float hi) {
     return pack_bf16x2(lo, hi);
 }
 
-// W consecutive bias values starting at column col (zero past N or if null).
-template <int W>
-__device__ __forceinline__ void load_bias(const float* bias, int col, int N, float (&b)[W]) {
-  if (bias && col + W <= N) {
-    const float4* p = reinterpret_cast<const float4*>(bias + col);
-#pragma unroll
-    for (int j = 0; j < W / 4; ++j) {
-      const float4 v = __ldg(p + j);
-      b[4 * j] = v.x;
-      b[4 * j + 1] = v.y;
-      b[4 * j + 2] = v.z;
-      b[4 * j + 3] = v.w;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < W; ++j) b[j] = (bias && col + j < N) ? __ldg(bias + col + j) : 0.0f;
-  }
-}
-
 // Implicit-GEMM convolution: number of M tiles and the pixel block of one.
 __host__ __device__ __forceinline__ int conv_mtiles(const GemmArgs& a) {
   return ((a.cv_wo + a.cv_bw - 1) / a.cv_bw) * ((a.cv_ho + a.cv_bh - 1) / a.cv_bh) *
@@ -145,25 +141,34 @@ __device__ __forceinline__ void conv_tile(const GemmArgs& a, int mtile, int& b0,
   b0 = (r / ty) * a.cv_nb;
 }
 
-// Walks this CTA's sequence of (tile, chunk) pairs, skipping chunks past N.
+// Walks the chunks of one epilogue warp group over this CTA's tiles. The
+// chunks of all tiles form one sequence (cols(t) of them in tile t); group g
+// takes every third one, so that tiles of a single chunk go round.
+__device__ __forceinline__ int first_chunk(int g, int before) { return (g + GROUPS - before) % GROUPS; }
 struct ChunkIter {
-  int t, c;
+  int t, c, before;  // tile, chunk in it, number of chunks before the tile (mod GROUPS)
   bool valid;
-  int stride;
-  __device__ __forceinline__ void init(int tiles, int start, int step) {
-    t = start;
-    stride = step;
-    c = 0;
-    valid = t < tiles;
-  }
-  __device__ __forceinline__ void advance(int tiles, int nt, int bn, int cw, int N) {
-    const int n0 = (t % nt) * bn;
-    ++c;
-    if (c * cw >= bn || n0 + c * cw >= N) {
-      c = 0;
+  template <class Cols>
+  __device__ __forceinline__ void settle(int tiles, int stride, int g, Cols&& cols) {
+    while (valid && c >= cols(t)) {
+      before = (before + cols(t)) % GROUPS;
       t += stride;
+      c = first_chunk(g, before);
       valid = t < tiles;
     }
+  }
+  template <class Cols>
+  __device__ __forceinline__ void init(int tiles, int start, int stride, int g, Cols&& cols) {
+    t = start;
+    before = 0;
+    c = g;
+    valid = t < tiles;
+    settle(tiles, stride, g, cols);
+  }
+  template <class Cols>
+  __device__ __forceinline__ void advance(int tiles, int stride, int g, Cols&& cols) {
+    c += GROUPS;
+    settle(tiles, stride, g, cols);
   }
 };
 
@@ -196,14 +201,16 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   uint64_t* tfull = bars + 2 * MAX_STAGES;
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
-  uint64_t* rfull = drain + 1;  // MAX_CBUFS residual-landed barriers
-  uint64_t* bfull = rfull + MAX_CBUFS;  // resident B landed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bfull + 1);
+  uint64_t* bfull = drain + 1;  // resident B landed
+  uint64_t* rfull = bfull + 1;  // residual landed: MAX_CBUFS barriers per epilogue warp
+  float* sbias = reinterpret_cast<float*>(rfull + EPI_WARPS * MAX_CBUFS);  // 32 values per epilogue warp
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sbias + 32 * EPI_WARPS);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int M = args.M, N = args.N, bn = args.bn;
   constexpr int TM = PAIR ? 2 * BM : BM;  // rows per tile
-  const int mt = args.conv ? conv_mtiles(args) : (M + TM - 1) / TM, nt = (N + bn - 1) / bn;
+  // (a pair takes two consecutive pixel blocks of a convolution)
+  const int mt = args.conv ? (conv_mtiles(args) + PAIR) / (1 + PAIR) : (M + TM - 1) / TM, nt = (N + bn - 1) / bn;
   // split-K (fp32 partial outputs only): tile t covers output tile
   // t % (mt * nt) and k-block range t / (mt * nt) of ks. Every other
   // epilogue has ks = 1 at compile time and no division on its tile path.
@@ -223,12 +230,13 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], (PAIR ? 2 : 1) * (TR::tma ? EPI_THREADS / 32 : 4));
+      mbar_init(&tempty[a], (PAIR ? 2 : 1) * (TR::tma ? EPI_WARPS : 4));
     }
     mbar_init(drain, 1);
-    for (int e = 0; e < MAX_CBUFS; ++e) mbar_init(&rfull[e], 1);
+    if constexpr (TR::resid)
+      for (int e = 0; e < EPI_WARPS * MAX_CBUFS; ++e) mbar_init(&rfull[e], 1);
     mbar_init(bfull, 1);
-    tmem_slot[1] = 0;  // the epilogue's fail flag
+    for (int i = 0; i < GROUPS; ++i) tmem_slot[1 + i] = 0;  // the convolution epilogue groups' fail flags
     fence_barrier_init();
   }
   if (warp == 0) {
@@ -269,7 +277,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   // lane 0 of each) that take alternate k-blocks: issuing one 4-D box load
   // occupies its warp for ~0.26 us, longer than the tensor core spends on a
   // narrow k-block.
-  const int nprod = (!PAIR && args.conv && static_cast<int>(blockDim.x) == THREADS_CONV) ? 2 : 1;
+  const int nprod = (args.conv && static_cast<int>(blockDim.x) == THREADS_CONV) ? 2 : 1;
   if (warp == 0 || warp == THREADS / 32) {
     // ------------------------------------------------------------ producer
     const int pid = warp == 0 ? 0 : 1;
@@ -280,8 +288,8 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
       long last_mine = -1;  // the last k-block this thread issued
       bool ok = true;
       // pair: the even CTA's full barrier counts both CTAs' bytes
-      const uint32_t bytes = PAIR ? 2 * (A_STAGE + (bn / 2) * BK * 2)
-                                  : (args.conv ? args.cv_a_bytes : A_STAGE) + (bres ? 0 : NB * bn * bke * 2);
+      const uint32_t a_bytes = args.conv ? args.cv_a_bytes : A_STAGE;
+      const uint32_t bytes = PAIR ? 2 * (a_bytes + (bn / 2) * BK * 2) : a_bytes + (bres ? 0 : NB * bn * bke * 2);
       const bool b_loaded = bres && t_start < tiles && pid == 0;
       if (b_loaded) {  // all of W, once: nk k-blocks of the single N tile
         mbar_expect_tx(bfull, static_cast<uint32_t>(nk) * bn * bke * 2);
@@ -314,7 +322,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         int cb0 = 0, cy0 = 0, cx0 = 0;  // implicit conv: first image, output row and column of the tile
         int cg = 0, kx = 0, ky = 0;     // implicit conv: the k-block's channel group and tap, advanced in step
         if (args.conv) {
-          conv_tile(args, m_tile(args, tq / nt, mt), cb0, cy0, cx0);
+          conv_tile(args, m_tile(args, tq / nt, mt) * (1 + PAIR) + rank, cb0, cy0, cx0);
           const int tap = kb0 / args.cv_cgroups;
           cg = kb0 - tap * args.cv_cgroups;
           ky = tap / args.cv_ks;
@@ -322,14 +330,18 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
         for (int kb = kb0; kb < kb1; ++kb, ++seq) {
           if (mine(seq)) {
-            if (!(PAIR ? mbar_wait_cluster(&empty[stage], phase ^ 1) : mbar_wait(&empty[stage], phase ^ 1))) {
+            if (!mbar_wait(&empty[stage], phase ^ 1)) {
               ok = false;
               break;
             }
             if constexpr (PAIR) {
               const uint32_t full_lead = cluster_map(smem_addr(&full[stage]), 0);
               if (leader) mbar_expect_tx(&full[stage], bytes);
-              tma_load_2d_pair(sA + stage * A_STAGE, &tmA, full_lead, kb * BK, m0);
+              if (args.conv)
+                tma_load_4d_pair(sA + stage * A_STAGE, &tmA, full_lead, cg * BK,
+                                 cx0 * args.cv_stride - args.cv_pad + kx, cy0 * args.cv_stride - args.cv_pad + ky, cb0);
+              else
+                tma_load_2d_pair(sA + stage * A_STAGE, &tmA, full_lead, kb * BK, m0);
               tma_load_2d_pair(sB + stage * BSTG, &tmB, full_lead, kb * BK, n0 + rank * (bn / 2));
             } else {
               const bool armed = seq < pre;  // this stage's weights were requested before the wait
@@ -370,7 +382,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         if (!mine(q) || q > last_mine) continue;
         const int st = static_cast<int>(q % S);
         const uint32_t ph = static_cast<uint32_t>((q / S) & 1);
-        PAIR ? mbar_wait_cluster(&full[st], ph) : mbar_wait(&full[st], ph);
+        mbar_wait(&full[st], ph);
       }
       if (b_loaded) mbar_wait(bfull, 0);
     }
@@ -387,7 +399,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
       for (int t = t_start; t < tiles && ok; t += t_stride, ++local) {
         const int acc = local & 1;
         const uint32_t use = static_cast<uint32_t>(local >> 1);
-        if (!(PAIR ? mbar_wait_cluster(&tempty[acc], (use & 1) ^ 1) : mbar_wait(&tempty[acc], (use & 1) ^ 1))) {
+        if (!mbar_wait(&tempty[acc], (use & 1) ^ 1)) {
           ok = false;
           break;
         }
@@ -400,7 +412,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
         const int kb0 = kSplit ? (t / mn_tiles) * nk / ks : 0, kb1 = kSplit ? (t / mn_tiles + 1) * nk / ks : nk;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!(PAIR ? mbar_wait_cluster(&full[stage], phase) : mbar_wait(&full[stage], phase))) {
+          if (!mbar_wait(&full[stage], phase)) {
             ok = false;
             break;
           }
@@ -457,157 +469,196 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   } else if constexpr (TR::tma) {
     // ------------------------------------------------------------ TMA-store epilogue
     constexpr int CW = TR::cw;
-    constexpr int NG = EPI_THREADS / 128;   // warp groups sharing each chunk
-    constexpr int HW = CW / NG;             // columns of a chunk handled by one thread
-    constexpr int NC = HW * (TR::f32 ? 4 : 2) / 16;  // 16-byte pieces per thread
-    const int q = warp & 3;                 // TMEM lane quarter
-    const int g = (warp - 2) >> 2;          // warp group: which part of each chunk
-    const int r = q * 32 + lane;            // row within the tile
-    const bool elected = threadIdx.x == 64;
+    const int ew = warp - 2;
+    const int q = warp & 3;       // TMEM lane quarter: rows 32q .. 32q + 31 of the tile
+    const int g = ew >> 2;        // takes every third chunk
     const int cpt = bn / CW;
     const uint32_t row_tm = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
-    // Every epilogue thread waits on the accumulator and residual barriers
-    // itself (no barrier round just to share one thread's wait); a wait that
-    // gives up raises `fail`. The flag is read only right after the chunk's
-    // named barrier, where all threads see the same value, so the 512
-    // threads leave together and the barrier is never left one arrival short.
-    volatile int* fail = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    ChunkIter pf;  // residual prefetch iterator (elected thread only)
-    pf.init(tiles, t_start, t_stride);
-    long loads = 0, consumed = 0, stored = 0;
+    auto piece = [&](int e) { return sC + ((g * E + e) * 4 + q) * WBUF; };  // a group's four pieces are one 16 KB chunk
+    auto cols = [&](int t) {
+      const int left = (N - (t % nt) * bn + CW - 1) / CW;
+      return left < cpt ? left : cpt;
+    };
+    auto row0 = [&](int t) { return m_tile(args, t / nt, mt) * TM + rank * BM; };
+    // Warps work on their own: each reads its 32 rows of its chunks, writes
+    // them to its own staging pieces and stores them with its own 32-row TMA
+    // boxes; the only hand-offs are the accumulator barriers. (Convolution
+    // tiles are pixel blocks whose quarters are no boxes: the four warps of a
+    // group meet at a named barrier and one stores the 128-row chunk.)
+    // A convolution warp whose wait gave up tells its group, which leaves
+    // together after its next barrier.
+    volatile uint32_t* fail = tmem_slot + 1 + g;
+    uint64_t* rf = rfull + ew * MAX_CBUFS;
+    float* sb = sbias + 32 * ew;
+    ChunkIter pf;  // residual prefetch (lane 0)
+    long loads = 0, consumed = 0;
+    auto fetch = [&](int e) {
+      mbar_expect_tx(&rf[e], WBUF);
+      tma_load_2d(piece(e), &tmR, &rf[e], (pf.t % nt) * bn + pf.c * CW, resid_row(args, row0(pf.t)) + q * 32);
+      pf.advance(tiles, t_stride, g, cols);
+      ++loads;
+    };
     if constexpr (TR::resid) {
-      if (elected) {
-        for (int e = 0; e < E && pf.valid; ++e) {
-          mbar_expect_tx(&rfull[e], CBUF);
-          tma_load_2d(sC + e * CBUF, &tmR, &rfull[e], (pf.t % nt) * bn + pf.c * CW,
-                      resid_row(args, m_tile(args, pf.t / nt, mt) * TM + rank * BM));
-          pf.advance(tiles, nt, bn, CW, N);
-          ++loads;
-        }
+      if (lane == 0) {
+        pf.init(tiles, t_start, t_stride, g, cols);
+        for (int e = 0; e < E && pf.valid; ++e) fetch(e);
       }
     }
-    int e = 0;
+    int e = 0, before = 0;
     uint32_t rph = 0;
     bool ok = true;
     int local = 0;
     for (int t = t_start; t < tiles && ok; t += t_stride, ++local) {
       const int acc = local & 1;
       const uint32_t use = static_cast<uint32_t>(local >> 1);
-      if (!(PAIR ? mbar_wait_cluster(&tfull[acc], use & 1) : mbar_wait(&tfull[acc], use & 1))) *fail = 1;
-      tc_fence_after();
-      const int m0 = m_tile(args, t / nt, mt) * TM + rank * BM, n0 = (t % nt) * bn;
-      const uint32_t acc_tm = row_tm + acc * MAX_BN;
-      int nvalid = 0;
-      while (nvalid < cpt && n0 + nvalid * CW < N) ++nvalid;
-      for (int c = 0; c < nvalid; ++c) {
-        uint8_t* buf = sC + e * CBUF;
-        uint8_t* rowp = buf + r * 128;
-        if constexpr (TR::resid) {
-          if (!mbar_wait(&rfull[e], rph)) *fail = 1;
-          ++consumed;
+      const int m0 = row0(t), n0 = (t % nt) * bn, nvalid = cols(t);
+      int c = first_chunk(g, before);
+      before = (before + nvalid) % GROUPS;
+      // Each chunk's bias is requested a chunk ahead (before the accumulator
+      // wait for the first), one column per lane, and broadcast from shared
+      // memory: reading it where it is used, every thread every column, left
+      // the warp waiting on the loaded L2 path for a third of the chunk.
+      float nb[CW / 32];
+      auto bias_of = [&](int chunk) {
+#pragma unroll
+        for (int h = 0; h < CW / 32; ++h) {
+          const int k = n0 + chunk * CW + 32 * h + lane;
+          nb[h] = args.bias && k < N ? __ldg(args.bias + k) : 0.0f;
         }
-        {
-          // this thread: row r, columns [g*HW, g*HW + HW) of the chunk = the
-          // 16-byte pieces NC*g .. NC*g + NC-1 of the 128-byte staging row
-          uint32_t v[HW];
-          if (nk > 0) {
-            if constexpr (HW == 32)
-              tmem_ld_32x32b_x32(acc_tm + c * CW + g * HW, v);
-            else if constexpr (HW == 16)
-              tmem_ld_16(acc_tm + c * CW + g * HW, v);
-            else
-              tmem_ld_8(acc_tm + c * CW + g * HW, v);
-            tmem_ld_wait();
-          } else {
+      };
+      bias_of(c);
+      ok = __all_sync(0xffffffffu, mbar_wait(&tfull[acc], use & 1));
+      if (!ok) {
+        if (!args.conv) break;
+        *fail = 1;
+        ok = true;
+      }
+      tc_fence_after();
+      const uint32_t acc_tm = row_tm + acc * MAX_BN;
+      auto release = [&] {  // this warp's last TMEM read of the tile is done
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if constexpr (PAIR)
+            mbar_arrive_cluster(cluster_map(smem_addr(&tempty[acc]), 0));  // the even CTA issues the MMAs
+          else
+            mbar_arrive(&tempty[acc]);
+        }
+      };
+      if (c >= nvalid) release();
+      for (; c < nvalid; c += GROUPS) {
+        uint8_t* const rowp = piece(e) + lane * 128;
+        const int col = n0 + c * CW;
+        uint32_t v[CW / 32][32];
+        float bl[CW / 32];
+        if (nk > 0) tmem_ld_32x32b_x32(acc_tm + c * CW, v[0]);
 #pragma unroll
-            for (int j = 0; j < HW; ++j) v[j] = 0u;
-          }
-          if (c == nvalid - 1) {  // last TMEM read of this tile
-            tc_fence_before();
-            if (lane == 0) {
-              if constexpr (PAIR)
-                mbar_arrive_cluster(cluster_map(smem_addr(&tempty[acc]), 0));  // the even CTA issues the MMAs
-              else
-                mbar_arrive(&tempty[acc]);
+        for (int h = 0; h < CW / 32; ++h) bl[h] = nb[h];
+        if (c + GROUPS < nvalid) bias_of(c + GROUPS);
+        sb[lane] = bl[0];
+        __syncwarp();
+        if (nk > 0) {
+          tmem_ld_wait();
+          if constexpr (CW == 64) tmem_ld_32x32b_x32(acc_tm + c * CW + 32, v[1]);  // in flight while v[0] is worked on
+        } else {
+#pragma unroll
+          for (int j = 0; j < CW; ++j) v[j / 32][j & 31] = 0u;
+        }
+        if (CW == 32 && c + GROUPS >= nvalid) release();
+        if constexpr (TR::resid) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&rf[e], rph));
+          if (!ok) break;
+          ++consumed;
+        } else {
+          // the piece is free once the store that last read it (E chunks ago) has done so
+          if (lane == 0) E == 1 ? bulk_wait_read<0>() : bulk_wait_read<1>();
+          if (args.conv)
+            named_bar_sync(1 + g, 128);  // (one warp issues the group's stores)
+          else
+            __syncwarp();
+        }
+        // 16-byte pieces of the 128-byte staging row, swizzled as the TMA box is
+        if constexpr (TR::f32) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float4* p = reinterpret_cast<float4*>(rowp + ((j ^ (lane & 7)) << 4));
+            const float4 bb = reinterpret_cast<const float4*>(sb)[j];
+            float2 lo = add2(make_float2(__uint_as_float(v[0][4 * j]), __uint_as_float(v[0][4 * j + 1])),
+                             make_float2(bb.x, bb.y));
+            float2 hi = add2(make_float2(__uint_as_float(v[0][4 * j + 2]), __uint_as_float(v[0][4 * j + 3])),
+                             make_float2(bb.z, bb.w));
+            if constexpr (TR::resid) {  // X_old arrived by TMA into the same place
+              const float4 o = *p;
+              lo = add2(make_float2(o.x, o.y), lo);
+              hi = add2(make_float2(o.z, o.w), hi);
             }
+            *p = make_float4(lo.x, lo.y, hi.x, hi.y);
           }
-          float bb[HW];
-          load_bias<HW>(args.bias, n0 + c * CW + g * HW, N, bb);
-          if constexpr (TR::f32) {
-            // X_old arrived by TMA into the same swizzled row
+        } else {
 #pragma unroll
-            for (int j = 0; j < NC; ++j) {
-              float4* p = reinterpret_cast<float4*>(rowp + (((NC * g + j) ^ (r & 7)) << 4));
-              float4 o = *p;
-              o.x += __uint_as_float(v[4 * j]) + bb[4 * j];
-              o.y += __uint_as_float(v[4 * j + 1]) + bb[4 * j + 1];
-              o.z += __uint_as_float(v[4 * j + 2]) + bb[4 * j + 2];
-              o.w += __uint_as_float(v[4 * j + 3]) + bb[4 * j + 3];
-              *p = o;
+          for (int h = 0; h < 2; ++h) {
+            if (h == 1) {
+              __syncwarp();
+              sb[lane] = bl[1];
+              __syncwarp();
+              if (nk > 0) tmem_ld_wait();
+              if (c + GROUPS >= nvalid) release();
             }
-          } else if constexpr (TR::resid16) {
-            // the residual's 8 values arrived by TMA into this 16-byte piece
 #pragma unroll
-            for (int j = 0; j < NC; ++j) {
-              uint4* p = reinterpret_cast<uint4*>(rowp + (((NC * g + j) ^ (r & 7)) << 4));
-              const uint4 rv = *p;
-              const uint32_t rw[4] = {rv.x, rv.y, rv.z, rv.w};
-              uint32_t ow[4];
+            for (int j = 0; j < 4; ++j) {
+              uint4* p = reinterpret_cast<uint4*>(rowp + (((4 * h + j) ^ (lane & 7)) << 4));
+              uint32_t rw[4] = {0u, 0u, 0u, 0u}, ow[4];
+              if constexpr (TR::resid16) {  // the residual's 8 values arrived by TMA
+                const uint4 rv = *p;
+                rw[0] = rv.x, rw[1] = rv.y, rw[2] = rv.z, rw[3] = rv.w;
+              }
+              const float4 b4[2] = {reinterpret_cast<const float4*>(sb)[2 * j],
+                                    reinterpret_cast<const float4*>(sb)[2 * j + 1]};
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
-                const float2 rf = unpack_in<EPI>(rw[i]);
-                ow[i] = pack_out<EPI>(epi_act<EPI>(__uint_as_float(v[8 * j + 2 * i]) + bb[8 * j + 2 * i] + rf.x),
-                                      epi_act<EPI>(__uint_as_float(v[8 * j + 2 * i + 1]) + bb[8 * j + 2 * i + 1] +
-                                                   rf.y));
+                const int k = 8 * j + 2 * i;
+                const float2 bb = i & 1 ? make_float2(b4[i >> 1].z, b4[i >> 1].w)
+                                        : make_float2(b4[i >> 1].x, b4[i >> 1].y);
+                float2 x = add2(make_float2(__uint_as_float(v[h][k]), __uint_as_float(v[h][k + 1])), bb);
+                if constexpr (TR::resid16) x = add2(x, unpack_in<EPI>(rw[i]));
+                x = epi_act2<EPI>(x);
+                ow[i] = pack_out<EPI>(x.x, x.y);
               }
               *p = make_uint4(ow[0], ow[1], ow[2], ow[3]);
             }
-          } else {
-#pragma unroll
-            for (int j = 0; j < NC; ++j) {
-              uint4 pk;
-              pk.x = pack_out<EPI>(epi_act<EPI>(__uint_as_float(v[8 * j + 0]) + bb[8 * j + 0]),
-                                 epi_act<EPI>(__uint_as_float(v[8 * j + 1]) + bb[8 * j + 1]));
-              pk.y = pack_out<EPI>(epi_act<EPI>(__uint_as_float(v[8 * j + 2]) + bb[8 * j + 2]),
-                                 epi_act<EPI>(__uint_as_float(v[8 * j + 3]) + bb[8 * j + 3]));
-              pk.z = pack_out<EPI>(epi_act<EPI>(__uint_as_float(v[8 * j + 4]) + bb[8 * j + 4]),
-                                 epi_act<EPI>(__uint_as_float(v[8 * j + 5]) + bb[8 * j + 5]));
-              pk.w = pack_out<EPI>(epi_act<EPI>(__uint_as_float(v[8 * j + 6]) + bb[8 * j + 6]),
-                                 epi_act<EPI>(__uint_as_float(v[8 * j + 7]) + bb[8 * j + 7]));
-              *reinterpret_cast<uint4*>(rowp + (((NC * g + j) ^ (r & 7)) << 4)) = pk;
-            }
           }
         }
-        fence_async_smem();
-        // The previous chunk's store (issued a whole chunk ago) must have read
-        // its buffer before anyone passes this barrier: after it, that buffer
-        // is written by the next chunk (E = 2) or refilled by the prefetch.
-        if (elected) bulk_wait_read_all();
-        named_bar_sync(1, EPI_THREADS);
-        if (*fail) {
-          ok = false;
-          break;
-        }
-        if (elected) {
-          if (args.conv) {
+        fence_async_smem();  // (the barriers below also order this chunk's bias reads before the next one's write)
+        if (args.conv) {
+          const bool first = q == 0 && lane == 0;  // (its piece is the chunk's first)
+          named_bar_sync(1 + g, 128);
+          if (*fail) {
+            ok = false;
+            break;
+          }
+          if (first) {
             int cb0, cy0, cx0;
-            conv_tile(args, m_tile(args, t / nt, mt), cb0, cy0, cx0);
-            tma_store_4d(&tmC, buf, n0 + c * CW, cx0, cy0, cb0);
-          } else {
-            tma_store_2d(&tmC, buf, n0 + c * CW, m0);
+            conv_tile(args, m_tile(args, t / nt, mt) * (1 + PAIR) + rank, cb0, cy0, cx0);
+            if (cb0 < args.cv_batch) tma_store_4d(&tmC, piece(e), col, cx0, cy0, cb0);  // (a pair's last block may be none)
+            bulk_commit();
           }
-          bulk_commit();  // stays in flight while the next chunk is computed
-          if constexpr (TR::resid) {
-            if (stored > 0 && pf.valid) {
-              const int ep = e == 0 ? E - 1 : e - 1;  // buffer of the previous chunk
-              mbar_expect_tx(&rfull[ep], CBUF);
-              tma_load_2d(sC + ep * CBUF, &tmR, &rfull[ep], (pf.t % nt) * bn + pf.c * CW,
-                          resid_row(args, m_tile(args, pf.t / nt, mt) * TM + rank * BM));
-              pf.advance(tiles, nt, bn, CW, N);
-              ++loads;
+        } else {
+          __syncwarp();
+          if (lane == 0) {
+            if constexpr (TR::resid)
+              if (E > 1) bulk_wait_read<0>();  // the previous chunk's store: its piece is refilled below
+            if (m0 + q * 32 < M) {
+              if constexpr (EPI == EPI_BIAS_ADD_F32)
+                tma_add_2d(&tmC, piece(e), col, m0 + q * 32);
+              else
+                tma_store_2d(&tmC, piece(e), col, m0 + q * 32);
+            }
+            bulk_commit();
+            if constexpr (TR::resid) {
+              if (E == 1) bulk_wait_read<0>();
+              if ((E == 1 || consumed > 1) && pf.valid) fetch(e == 0 ? E - 1 : e - 1);
             }
           }
-          ++stored;
         }
         if (++e == E) {
           e = 0;
@@ -615,20 +666,19 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
       }
     }
-    if (!ok && elected) record_status(args.status, ELASTO_ERR_TIMEOUT);
-    if (elected) {
+    if (lane == 0) {
+      if (!ok) record_status(args.status, ELASTO_ERR_TIMEOUT);
       bulk_wait_all();
-      if constexpr (TR::resid) {
-        // Residual loads issued for chunks never consumed (only on the abort
-        // path): let them land before the CTA releases its shared memory.
+      // Residual loads issued for chunks never consumed (only on the abort
+      // path): let them land before the CTA releases its shared memory.
+      if constexpr (TR::resid)
         for (long i = consumed; i < loads; ++i) {
-          mbar_wait(&rfull[e], rph);
+          mbar_wait(&rf[e], rph);
           if (++e == E) {
             e = 0;
             rph ^= 1;
           }
         }
-      }
     }
   } else {
     // ------------------------------------------------------------ transpose epilogue
@@ -787,7 +837,7 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
   a.cv_batch = M;  // implicit convolutions: M counts images
   const int nt = (a.N + a.bn - 1) / a.bn;
   if constexpr (PAIR) {
-    static int max_clusters[64] = {0};
+    static int max_clusters[64] = {0};  // (one CTA per SM by shared memory, whatever its threads)
     int dev = 0;
     cudaGetDevice(&dev);
     cudaLaunchConfig_t cfg{};
@@ -798,7 +848,7 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_pdl
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.blockDim = dim3(THREADS);
+    cfg.blockDim = dim3(a.conv ? THREADS_CONV : THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -810,7 +860,7 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
       if (e != cudaSuccess || n <= 0) return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
       max_clusters[dev] = n;
     }
-    const int tiles = ((M + 2 * BM - 1) / (2 * BM)) * nt;
+    const int tiles = (a.conv ? (conv_mtiles(a) + 1) / 2 : (M + 2 * BM - 1) / (2 * BM)) * nt;
     const int clusters = tiles < max_clusters[dev] ? tiles : max_clusters[dev];
     cfg.gridDim = dim3(2 * clusters);
     cfg.numAttrs = 2;
@@ -840,6 +890,7 @@ cudaError_t gemm_init_attributes() {
   SET_ATTR(EPI_BIAS_BF16)
   SET_ATTR(EPI_BIAS_GELU_BF16)
   SET_ATTR(EPI_BIAS_RESID_F32)
+  SET_ATTR(EPI_BIAS_ADD_F32)
   SET_ATTR(EPI_BIAS_F32)
   SET_ATTR(EPI_BIAS_RELU_BF16)
   SET_ATTR(EPI_BIAS_RESID_RELU_BF16)
@@ -851,30 +902,78 @@ cudaError_t gemm_init_attributes() {
   SET_ATTR_PAIR(EPI_BIAS_BF16)
   SET_ATTR_PAIR(EPI_BIAS_GELU_BF16)
   SET_ATTR_PAIR(EPI_BIAS_RESID_F32)
+  SET_ATTR_PAIR(EPI_BIAS_ADD_F32)
   SET_ATTR_PAIR(EPI_BIAS_RELU_BF16)
 #undef SET_ATTR
 #undef SET_ATTR_PAIR
   return cudaSuccess;
 }
 
-int gemm_pick_bn(int M, int N, int step, bool pair) {
-  // Estimated time ~ waves x (bn + fixed per-tile overhead); ties prefer wider tiles.
-  const int sms = num_sms() > 0 ? num_sms() : 148;
-  const int units = pair ? sms / 2 : sms;  // concurrent tile workers
-  const int mt = (M + (pair ? 2 * BM : BM) - 1) / (pair ? 2 * BM : BM);
-  int best = 256;
-  long best_cost = -1;
-  for (int bn = 256; bn >= step; bn -= step) {
-    const long tiles = static_cast<long>(mt) * ((N + bn - 1) / bn);
-    const long waves = (tiles + units - 1) / units;
-    const long cost = waves * (bn + 32);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = bn;
-    }
-  }
-  return best;
+namespace {
+
+bool is_resid16(int epi) { return epi == EPI_BIAS_RESID_RELU_BF16 || epi == EPI_BIAS_RESID_RELU_F16; }
+
+// Bytes of one ring stage (A tile and the CTA's part of the B tile).
+int stage_bytes(int bn, bool pair, int planes) { return A_STAGE + (pair ? bn / 2 : planes * bn) * BK * 2; }
+
+// A GEMM (or implicit convolution, M = 128 rows per pixel block) to choose a
+// tiling for.
+struct Problem {
+  int M, N, K, planes, epi;
+  bool conv;
+  int sms;
+};
+
+// Estimated nanoseconds of one launch with 128-row (pair: 256-row) x bn tiles.
+// A k-block costs its MMAs or the delivery of its operands to shared memory,
+// whichever is longer; a tile its k-blocks or its epilogue, which overlap; the
+// last tile's epilogue is exposed, and clusters take longer to start. The
+// constants are fitted to launches of 197 to 50432 rows.
+double tile_cost(const Problem& p, int bn, bool pair) {
+  const int units = pair ? p.sms / 2 : p.sms, rows = pair ? 2 * BM : BM;
+  const long tiles = static_cast<long>((p.M + rows - 1) / rows) * ((p.N + bn - 1) / bn);
+  const long waves = (tiles + units - 1) / units;
+  double load = stage_bytes(bn, pair, p.planes) / 126.0, mma = p.planes * (130.0 + 0.9 * bn);
+  if (p.conv) load = std::max(load, 280.0);  // 4-D boxes
+  const double main_loop = ((p.K + BK - 1) / BK) * std::max(load, mma);
+  const bool f32 = p.epi == EPI_BIAS_RESID_F32 || p.epi == EPI_BIAS_ADD_F32;
+  const double epilogue = 400.0 + bn * (f32 ? 8.0 : p.epi == EPI_BIAS_GELU_BF16 ? 9.0 : 6.0);
+  return waves * (std::max(main_loop, epilogue) + 100.0) + epilogue + (pair ? 800.0 : 0.0);
 }
+
+// The tiling with the least estimated time: N tile (a multiple of step) on
+// single CTAs or, where allowed, CTA pairs. Ties prefer single CTAs, then wider tiles.
+void choose_tile(const Problem& p, int step, bool pairs_allowed, int* bn, bool* pair) {
+  double best = -1.0;
+  for (int two = 0; two <= (pairs_allowed ? 1 : 0); ++two)
+    for (int b = 256; b >= step; b -= step) {
+      const double cost = tile_cost(p, b, two != 0);
+      if (best < 0.0 || cost < best) {
+        best = cost;
+        *bn = b;
+        *pair = two != 0;
+      }
+    }
+}
+
+}  // namespace
+
+namespace {
+
+// Splits the pool between the operand ring and the epilogue's staging pieces.
+// cbufs counts pieces per epilogue warp: 2 with a residual read through them
+// (its fetch depth), if that leaves 3 stages, else 1.
+bool ring_layout(GemmArgs* a, bool resid) {
+  const int stage = a->b_stage + A_STAGE;
+  for (int e = resid ? MAX_CBUFS : 1; e >= 1; --e) {
+    a->cbufs = e;
+    a->stages = std::min((POOL - e * CBUF) / stage, MAX_STAGES);
+    if (a->stages >= 3) break;
+  }
+  return a->stages >= 2 && a->cbufs >= 1 && a->cbufs <= MAX_CBUFS && a->stages * stage + a->cbufs * CBUF <= POOL;
+}
+
+}  // namespace
 
 elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, int N, int K, const float* bias,
                         void* out, int ldo, int epi, int* status, const bf16* W_lo, int M_hint, int ldw,
@@ -889,64 +988,58 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
     return ELASTO_ERR_UNSUPPORTED;
   }
   *p = GemmPlan{};
-  const bool resid16 = epi == EPI_BIAS_RESID_RELU_BF16 || epi == EPI_BIAS_RESID_RELU_F16;
-  const bool tma_out = epi == EPI_BIAS_BF16 || epi == EPI_BIAS_GELU_BF16 || epi == EPI_BIAS_RELU_BF16 ||
-                       epi == EPI_BIAS_RESID_F32 || epi == EPI_BIAS_RELU_F16 || epi == EPI_BIAS_F16 || resid16;
-  const bool f32_out = epi == EPI_BIAS_RESID_F32;
-  const bool has_resid = f32_out || resid16;
+  if (epi == EPI_BIAS_RESID_F32) epi = EPI_BIAS_ADD_F32;  // the residual is the output itself
+  const bool resid16 = is_resid16(epi);
+  const bool f32_out = epi == EPI_BIAS_ADD_F32;
+  const bool tma_out = epi != EPI_BIAS_F32;
   GemmArgs& a = p->args;
   a.f16 = (epi == EPI_BIAS_RELU_F16 || epi == EPI_BIAS_F16 || epi == EPI_BIAS_RESID_RELU_F16) ? 1 : 0;
   a.M = M_cap;
   a.N = N;
   a.K = K;
-  // CTA pairs for the TMA-store epilogues on problems with at least one
-  // 256-row tile and single-plane weights
-  // (long reductions only: with K = 768 the per-tile epilogue dominates and
-  // a single CTA per tile measured faster)
   const int Mt = (M_hint > 0 && M_hint < M_cap) ? M_hint : M_cap;  // rows the tiling is chosen for
-  const bool pair = tma_out && !W_lo && Mt >= 2 * BM && K >= 1536;
+  const int planes = W_lo ? 2 : 1;
+  // 16-bit staging chunks are 64 columns wide: their tiles are multiples of 64
+  const int step = (tma_out && !f32_out) ? 64 : 32;
+  const int sms = num_sms() > 0 ? num_sms() : 152;
+  // CTA pairs (256-row tiles, each CTA loading half of B): the TMA-store
+  // epilogues without a 16-bit residual, single-plane weights
+  bool pair = false;
+  a.bn = bn_force;
+  if (bn_force <= 0)
+    choose_tile({Mt, N, K, planes, epi, false, sms}, step, tma_out && !resid16 && !W_lo && Mt >= 2 * BM && K > 0, &a.bn,
+                &pair);
   a.pair = pair ? 1 : 0;
-  // bf16 staging chunks are 64 columns wide: their tiles are multiples of 64
-  a.bn = bn_force > 0 ? bn_force : gemm_pick_bn(Mt, N, (tma_out && !f32_out) ? 64 : 32, pair);
   // one B stage holds exactly the tile's rows (both planes); the freed bytes
   // become a deeper operand ring for narrow tiles
-  a.b_stage = pair ? (a.bn / 2) * BK * 2 : (W_lo ? 2 : 1) * a.bn * BK * 2;
+  a.b_stage = stage_bytes(a.bn, pair, planes) - A_STAGE;
   a.bias = bias;
   a.out = out;
   a.ldo = ldo;
   a.status = status;
-  a.b_planes = W_lo ? 2 : 1;
+  a.b_planes = planes;
+  // On a nearly idle chip reading X ahead, behind the main loop, beats the
+  // longer completion of a reduce-add.
+  const int rows = pair ? 2 * BM : BM;
+  const long tiles = static_cast<long>((Mt + rows - 1) / rows) * ((N + a.bn - 1) / a.bn);
+  if (epi == EPI_BIAS_ADD_F32 && 4 * tiles <= (pair ? sms / 2 : sms)) epi = EPI_BIAS_RESID_F32;
   p->epi = epi;
   if (tma_out) {
-    // residual GEMMs: 3 operand stages and 5 staging chunks fetched ahead;
-    // the others: 4 stages and 2 staging chunks.
-    // residual epilogues keep 5 staging chunks (residual rows fetched
-    // ahead), the others 2; the rest of the pool is operand ring
-    const int keep = has_resid ? 5 : 2;
-    a.stages = (POOL - keep * CBUF) / (A_STAGE + a.b_stage);
-    if (a.stages > MAX_STAGES) a.stages = MAX_STAGES;
-    if (a.stages < 2) a.stages = 2;
-    if (pair) a.stages = has_resid ? 5 : 6;  // tuned for the K >= 1536 reductions
-    a.cbufs = (POOL - a.stages * (A_STAGE + a.b_stage)) / CBUF;
-    if (a.cbufs > MAX_CBUFS) a.cbufs = MAX_CBUFS;
+    if (!ring_layout(&a, resid16 || epi == EPI_BIAS_RESID_F32)) {
+      set_error("gemm_plan: shared-memory layout does not fit");
+      return ELASTO_ERR_UNSUPPORTED;
+    }
     if (ldo % 8 != 0 ||
         !encode_tmap_2d(&p->tmC, out, ldo, M_cap, static_cast<uint64_t>(ldo) * (f32_out ? 4 : 2),
-                        f32_out ? 32 : 64, BM, f32_out)) {
+                        f32_out ? 32 : 64, 32, f32_out)) {
       set_error("gemm_plan: output tensor map (alignment or size)");
       return ELASTO_ERR_UNSUPPORTED;
     }
-    p->tmR = p->tmC;  // the residual is read from the output unless redirected
+    p->tmR = p->tmC;
   } else {
-    a.stages = (POOL - 4 * EPI_TILE * 4) / (A_STAGE + a.b_stage);
-    if (a.stages > 4) a.stages = 4;
+    a.stages = std::min((POOL - 4 * EPI_TILE * 4) / (A_STAGE + a.b_stage), 4);
     a.cbufs = 0;
-  }
-  {
-    // the operand ring, staging chunks (or transpose tiles) must fit the pool
-    const int bstg = a.b_stage;
-    const int tail = tma_out ? a.cbufs * CBUF : 4 * EPI_TILE * 4;
-    if (a.stages < 2 || a.stages > MAX_STAGES || a.cbufs > MAX_CBUFS || (tma_out && a.cbufs < 2) ||
-        a.stages * (A_STAGE + bstg) + tail > POOL) {
+    if (a.stages < 2) {
       set_error("gemm_plan: shared-memory layout does not fit");
       return ELASTO_ERR_UNSUPPORTED;
     }
@@ -1054,32 +1147,28 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
   const int rows = a.cv_bw * a.cv_bh * a.cv_nb;
   a.cv_a_bytes = rows * bke * 2;
   a.cv_batch = B_cap;
-  a.bn = gemm_pick_bn(conv_mtiles(a) * BM, N, 64, false);
+  const int Mt = conv_mtiles(a) * BM;
+  const Problem prob{Mt, N, a.K, 1, epi, true, num_sms() > 0 ? num_sms() : 152};
+  bool pair = false;
+  choose_tile(prob, 64, false, &a.bn, &pair);
   a.bias = bias;
   a.out = out;
   a.ldo = ldo;
   a.status = status;
   a.b_planes = 1;
   a.f16 = 1;
-  a.pair = 0;
   // one N tile whose whole W fits beside a 4-stage A ring: W is loaded once
   // per CTA and kept, instead of once per tile and k-block from L2
   const int nk = taps * cg;
   const int b_all = nk * a.bn * bke * 2;
-  a.b_resident = (N <= a.bn && 4 * A_STAGE + b_all + 2 * CBUF <= POOL) ? 1 : 0;
-  if (a.b_resident) {
-    a.b_stage = a.bn * bke * 2;  // one k-block of W
-    a.stages = (POOL - 2 * CBUF - b_all) / A_STAGE;
-    if (a.stages > MAX_STAGES) a.stages = MAX_STAGES;
-    a.cbufs = (POOL - a.stages * A_STAGE - b_all) / CBUF;
-  } else {
-    a.b_stage = a.bn * BK * 2;
-    a.stages = (POOL - 2 * CBUF) / (A_STAGE + a.b_stage);
-    if (a.stages > MAX_STAGES) a.stages = MAX_STAGES;
-    a.cbufs = (POOL - a.stages * (A_STAGE + a.b_stage)) / CBUF;
-  }
-  if (a.cbufs > MAX_CBUFS) a.cbufs = MAX_CBUFS;
-  if (a.cbufs < 2 || rows > BM || a.stages < 2) {
+  a.b_resident = (N <= a.bn && 4 * A_STAGE + b_all + CBUF <= POOL) ? 1 : 0;
+  if (!a.b_resident && !k16) choose_tile(prob, 64, true, &a.bn, &pair);
+  a.pair = pair ? 1 : 0;
+  a.b_stage = (a.pair ? a.bn / 2 : a.bn) * (a.b_resident ? bke : BK) * 2;
+  const int ring = POOL - (a.b_resident ? b_all : 0), stage = A_STAGE + (a.b_resident ? 0 : a.b_stage);
+  a.stages = std::min((ring - CBUF) / stage, MAX_STAGES);
+  a.cbufs = 1;
+  if (rows > BM || a.stages < 2) {
     set_error(std::string(who) + ": shared-memory layout does not fit");
     return ELASTO_ERR_UNSUPPORTED;
   }
@@ -1090,7 +1179,7 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
   const uint32_t ob[4] = {64u, uint32_t(a.cv_bw), uint32_t(a.cv_bh), uint32_t(a.cv_nb)};
   const uint32_t oe[4] = {1u, 1u, 1u, 1u};
   const bool wmap = k16 ? encode_tmap_2d_sw32(&p->tmB, Wt, a.K, N, uint64_t(a.K) * 2, 16, a.bn)
-                        : encode_tmap_2d(&p->tmB, Wt, a.K, N, uint64_t(a.K) * 2, BK, a.bn);
+                        : encode_tmap_2d(&p->tmB, Wt, a.K, N, uint64_t(a.K) * 2, BK, a.pair ? a.bn / 2 : a.bn);
   if (xb[1] > 256 || xb[2] > 256 || !encode_tmap_4d(&p->tmA, x, xd, xs, xb, xe, k16) || !wmap ||
       !encode_tmap_4d(&p->tmC, out, od, os, ob, oe)) {
     set_error(std::string(who) + ": cuTensorMapEncodeTiled failed (alignment or size)");
@@ -1163,8 +1252,8 @@ elasto_status gemm_plan_conv_rows(GemmPlan* p, const void* x, int B_cap, int Hp,
 }
 
 elasto_status gemm_set_residual_source(GemmPlan* p, const void* src, int M_cap, int row_period) {
-  const bool f32 = p && p->epi == EPI_BIAS_RESID_F32;
-  const bool r16 = p && (p->epi == EPI_BIAS_RESID_RELU_BF16 || p->epi == EPI_BIAS_RESID_RELU_F16);
+  const bool f32 = p && (p->epi == EPI_BIAS_ADD_F32 || p->epi == EPI_BIAS_RESID_F32);
+  const bool r16 = p && is_resid16(p->epi);
   if (!p || !p->valid || !(f32 || r16) || !src) {
     set_error("gemm_set_residual_source: needs a residual plan and a source");
     return ELASTO_ERR_INVALID_ARG;
@@ -1175,7 +1264,14 @@ elasto_status gemm_set_residual_source(GemmPlan* p, const void* src, int M_cap, 
   }
   p->args.resid_row_mod = row_period;
   const int ldo = p->args.ldo;
-  if (!encode_tmap_2d(&p->tmR, src, ldo, M_cap, static_cast<uint64_t>(ldo) * (f32 ? 4 : 2), f32 ? 32 : 64, BM,
+  if (f32) {  // the residual is read: stores instead of reduce-adds, and the staging depth to fetch it ahead
+    p->epi = EPI_BIAS_RESID_F32;
+    if (!ring_layout(&p->args, true)) {
+      set_error("gemm_set_residual_source: shared-memory layout does not fit");
+      return ELASTO_ERR_UNSUPPORTED;
+    }
+  }
+  if (!encode_tmap_2d(&p->tmR, src, ldo, M_cap, static_cast<uint64_t>(ldo) * (f32 ? 4 : 2), f32 ? 32 : 64, 32,
                       f32)) {
     set_error("gemm_set_residual_source: tensor map (alignment or size)");
     return ELASTO_ERR_UNSUPPORTED;
@@ -1197,6 +1293,7 @@ cudaError_t gemm_launch_main(const GemmPlan& p, int M, cudaStream_t s) {
     CASE_PAIR(EPI_BIAS_BF16)
     CASE_PAIR(EPI_BIAS_GELU_BF16)
     CASE_PAIR(EPI_BIAS_RESID_F32)
+    CASE_PAIR(EPI_BIAS_ADD_F32)
     CASE(EPI_BIAS_F32)
     CASE_PAIR(EPI_BIAS_RELU_BF16)
     CASE(EPI_BIAS_RESID_RELU_BF16)

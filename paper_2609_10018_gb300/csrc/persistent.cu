@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(PK_THREADS, 1)
           // row pieces -> this warp's staging box -> one TMA store of 32 rows
           // (rows past n and columns past N are clipped by the map)
           uint8_t* box = stg + (warp - 2) * PK_STG_WARP;
-          if (lane == 0) bulk_wait_read_all();  // the box's previous store has read it
+          if (lane == 0) bulk_wait_read<0>();  // the box's previous store has read it
           __syncwarp();
           stage_row(box, lane, ph.epi == PKE_PART ? half / 4 : half / 8, v);
           fence_async_smem();
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(PK_THREADS, 1)
             for (int q = 0; q < 16; ++q)
               o[q] = pack_bf16x2(__uint_as_float(o[2 * q]) * inv, __uint_as_float(o[2 * q + 1]) * inv);
             uint8_t* box = stg + (warp - 2) * PK_STG_WARP;
-            if (lane == 0) bulk_wait_read_all();
+            if (lane == 0) bulk_wait_read<0>();
             __syncwarp();
             stage_row(box, lane, 4, o);
             fence_async_smem();
