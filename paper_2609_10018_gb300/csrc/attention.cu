@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint64_t* drain = bars + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int w = heads * HD;
   const int tiles = n > QT ? 2 : 1;
   // items of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -117,13 +117,13 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = warp_uniform(static_cast<int>(*tmem_slot));
   pdl_wait();  // the set-up above overlapped the previous kernel's tail
   pdl_trigger();
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       tma_prefetch_desc(&tmQ);
       tma_prefetch_desc(&tmKV);
       const uint32_t bytes = tiles * Q_BYTES + 2 * n_pad * HD * 2;
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && nk > 0) {
+    if (nk > 0) {
       const uint32_t idesc_s = idesc_bf16_f32(QT, n_pad);
       const uint32_t idesc_o = idesc_bf16_f32(QT, HD, false, true);
       bool ok = true;
@@ -158,29 +158,29 @@ __global__ void __launch_bounds__(THREADS, 1)
       // read out (S overwrites the O columns of its tile region)
       auto issue_s = [&](int k, int t) -> bool {
         const int slot = k % ns;
-        if (t == 0 && !mbar_wait(&full[slot], (k / ns) & 1)) return false;
-        if (!mbar_wait(&o_empty[t], (k & 1) ^ 1)) return false;
+        if (t == 0 && !mbar_wait_warp(&full[slot], (k / ns) & 1)) return false;
+        if (!mbar_wait_warp(&o_empty[t], (k & 1) ^ 1)) return false;
         tc_fence_after();
         const uint32_t q0 = smem_addr(qbuf + (2 * t + (k & 1)) * Q_BYTES);
         const uint32_t k0 = smem_addr(kvbuf + slot * slot_bytes);
 #pragma unroll
         for (int kk = 0; kk < HD / 16; ++kk)
-          tc_mma(tmem + t * 256, sdesc_sw128(q0 + kk * 32, 16, 1024), sdesc_sw128(k0 + kk * 32, 16, 1024), idesc_s,
+          tc_mma_warp(tmem + t * 256, sdesc_sw128(q0 + kk * 32, 16, 1024), sdesc_sw128(k0 + kk * 32, 16, 1024), idesc_s,
                  kk != 0);
-        tc_commit(&s_full[t]);
-        if (t == tiles - 1) tc_commit(&q_empty[k & 1]);
+        tc_commit_warp(&s_full[t]);
+        if (t == tiles - 1) tc_commit_warp(&q_empty[k & 1]);
         return true;
       };
       // PV(k, t): needs P(k, t) in TMEM
       auto issue_pv = [&](int k, int t) -> bool {
-        if (!mbar_wait(&p_full[t], k & 1)) return false;
+        if (!mbar_wait_warp(&p_full[t], k & 1)) return false;
         tc_fence_after();
         const uint32_t v0 = smem_addr(kvbuf + (k % ns) * slot_bytes + slot_bytes / 2);
         for (int s = 0; s < n_pad / 16; ++s)
-          tc_mma_tmem_a(tmem + t * 256 + O_COL, tmem + t * 256 + 8 * s, sdesc_sw128(v0 + s * 16 * 128, 16384, 1024),
+          tc_mma_tmem_a_warp(tmem + t * 256 + O_COL, tmem + t * 256 + 8 * s, sdesc_sw128(v0 + s * 16 * 128, 16384, 1024),
                         idesc_o, s != 0);
-        tc_commit(&o_full[t]);
-        if (t == tiles - 1) tc_commit(&kv_empty[k % ns]);
+        tc_commit_warp(&o_full[t]);
+        if (t == tiles - 1) tc_commit_warp(&kv_empty[k % ns]);
         return true;
       };
       ok = issue_s(0, 0);
@@ -191,10 +191,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (ok && k + 1 < nk) ok = issue_s(k + 1, 0);
         if (ok && tiles == 2) ok = issue_pv(k, 1);
       }
-      if (!ok) record_status(status, ELASTO_ERR_TIMEOUT);
+      if (!ok && lane == 0) record_status(status, ELASTO_ERR_TIMEOUT);
       if (issued) {  // every MMA this thread issued has finished once `drain` completes
-        tc_commit(drain);
-        mbar_wait(drain, 0);
+        tc_commit_warp(drain);
+        mbar_wait_warp(drain, 0);
       }
     }
   } else {

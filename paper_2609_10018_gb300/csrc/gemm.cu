@@ -10,10 +10,11 @@
 //  - persistent grid, one CTA per SM (or one CTA pair per two SMs), static
 //    round-robin over 128 x bn tiles (N tile index fastest so the CTAs
 //    running together share A rows in L2; m_reverse runs the rows backwards);
-//  - warp 0 lane 0: TMA producer, ring of 128x64 (A) and bn x 64 (B) bf16 or
-//    f16 tiles with the 128-byte swizzle, one mbarrier pair per stage. W may
-//    instead be loaded once per CTA and kept (b_resident: one N tile);
-//  - warp 1 lane 0: issues tcgen05.mma (M=128, N=bn, K=16) into one of two
+//  - warp 0, one elected thread: TMA producer, ring of 128x64 (A) and bn x 64
+//    (B) bf16 or f16 tiles with the 128-byte swizzle, one mbarrier pair per
+//    stage. W may instead be loaded once per CTA and kept (b_resident: one N
+//    tile);
+//  - warp 1, as a whole: issues tcgen05.mma (M=128, N=bn, K=16) into one of two
 //    TMEM accumulators (2 x 256 fp32 columns), commits stages back to the
 //    producer and finished accumulators to the epilogue.
 //  - CTA pairs (cta_group::2, M = 256, each CTA holds half of B) where
@@ -70,8 +71,8 @@ constexpr int EPI_LD = 33;                  // padded row of the transpose tile
 constexpr int EPI_TILE = 32 * EPI_LD;       // floats per epilogue warp
 constexpr int TMEM_COLS = 512;
 constexpr size_t SMEM_BYTES = 1024 + POOL + 2048;
-static_assert((2 * MAX_STAGES + 6 + EPI_WARPS * MAX_CBUFS) * 8 + 32 * EPI_WARPS * 4 + 4 * (1 + GROUPS) <= 2048,
-              "barriers and bias");
+constexpr int BARS = 2 * MAX_STAGES + 6 + EPI_WARPS * MAX_CBUFS;  // mbarriers (the bias after them is read as float4)
+static_assert(BARS * 8 % 16 == 0 && BARS * 8 + 32 * EPI_WARPS * 4 + 4 * (1 + GROUPS) <= 2048, "barriers and bias");
 
 template <int EPI>
 struct EpiTraits {
@@ -203,10 +204,10 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   uint64_t* drain = tempty + 2;
   uint64_t* bfull = drain + 1;  // resident B landed
   uint64_t* rfull = bfull + 1;  // residual landed: MAX_CBUFS barriers per epilogue warp
-  float* sbias = reinterpret_cast<float*>(rfull + EPI_WARPS * MAX_CBUFS);  // 32 values per epilogue warp
+  float* sbias = reinterpret_cast<float*>(bars + BARS);  // 32 values per epilogue warp
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sbias + 32 * EPI_WARPS);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int M = args.M, N = args.N, bn = args.bn;
   constexpr int TM = PAIR ? 2 * BM : BM;  // rows per tile
   // (a pair takes two consecutive pixel blocks of a convolution)
@@ -218,9 +219,9 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   const int ks = kSplit && args.ksplit > 1 ? args.ksplit : 1;
   const int mn_tiles = mt * nt;
   const int tiles = mn_tiles * ks;
-  const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;  // this CTA's row half of a pair tile
-  const int t_start = PAIR ? static_cast<int>(cluster_id_x()) : static_cast<int>(blockIdx.x);
-  const int t_stride = PAIR ? static_cast<int>(cluster_count_x()) : static_cast<int>(gridDim.x);
+  const int rank = PAIR ? warp_uniform(static_cast<int>(cluster_ctarank())) : 0;  // this CTA's row half of a pair tile
+  const int t_start = PAIR ? warp_uniform(static_cast<int>(cluster_id_x())) : static_cast<int>(blockIdx.x);
+  const int t_stride = PAIR ? warp_uniform(static_cast<int>(cluster_count_x())) : static_cast<int>(gridDim.x);
   const bool leader = rank == 0;
 
   if (threadIdx.x == 0) {
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
       tmem_relinquish();
     }
   }
-  if (warp == 1 && lane == 0) {
+  if (warp == 1 && elect_one()) {
     if (nk > 0) {
       tma_prefetch_desc(&tmA);
       tma_prefetch_desc(&tmB);
@@ -263,25 +264,25 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   else
     __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = warp_uniform(static_cast<int>(*tmem_slot));
   // Everything above overlapped the previous kernel's tail. Every thread
   // waits for that kernel (pdl_wait) before its first access to data it may
   // write; the weights are not such data, so the producer thread starts
   // loading them first and waits after that.
-  if (!(warp == 0 && lane == 0 && nk > 0)) {
+  if (warp != 0 || nk == 0) {
     pdl_wait();
     pdl_trigger();
   }
 
-  // Implicit convolutions run two producer threads (warp 0 and warp 18,
-  // lane 0 of each) that take alternate k-blocks: issuing one 4-D box load
-  // occupies its warp for ~0.26 us, longer than the tensor core spends on a
-  // narrow k-block.
+  // Implicit convolutions run two producer threads (one of warp 0 and one of
+  // warp 14) that take alternate k-blocks: with one, the 4-D boxes pace narrow
+  // tiles (128 images of 56 x 56 x 16 -> 16 channels: 54 us with one, 48 us
+  // with two; the strided 128-channel 3x3 of stage 2: 37.4 and 35.6).
   const int nprod = (args.conv && static_cast<int>(blockDim.x) == THREADS_CONV) ? 2 : 1;
   if (warp == 0 || warp == THREADS / 32) {
     // ------------------------------------------------------------ producer
     const int pid = warp == 0 ? 0 : 1;
-    if (lane == 0 && pid < nprod && nk > 0) {
+    if (pid < nprod && nk > 0 && elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       long seq = 0;         // k-block sequence index over this CTA's tiles
@@ -296,8 +297,8 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         for (int kb = 0; kb < nk; ++kb) tma_load_2d(sB + kb * BSTG, &tmB, bfull, kb * bke, 0);
       }
       // the first tile's first S stages: armed and their weights requested
-      // before the wait (fresh stages: no empty-slot wait needed); thread 0
-      // issues these k-blocks
+      // before the wait (fresh stages: no empty-slot wait needed); the first
+      // producer issues these k-blocks
       int pre = 0;
       if (!PAIR && !bres && t_start < tiles) {
         const int tq = kSplit ? t_start % mn_tiles : t_start;
@@ -388,31 +389,33 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && leader) {
+    if (leader) {
       const uint32_t idesc = idesc_16_f32(TM, bn, args.f16 != 0);
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true, issued = false;
       // resident B: every tile's MMAs read it; wait for it once
-      if (bres && t_start < tiles && !mbar_wait(bfull, 0)) ok = false;
+      if (bres && t_start < tiles && !mbar_wait_warp(bfull, 0)) ok = false;
       int local = 0;
       for (int t = t_start; t < tiles && ok; t += t_stride, ++local) {
         const int acc = local & 1;
         const uint32_t use = static_cast<uint32_t>(local >> 1);
-        if (!mbar_wait(&tempty[acc], (use & 1) ^ 1)) {
+        if (!mbar_wait_warp(&tempty[acc], (use & 1) ^ 1)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t dtm = tmem_base + acc * MAX_BN;
         if (nk == 0) {
-          mbar_arrive(&tfull[acc]);
-          if constexpr (PAIR) mbar_arrive_cluster(cluster_map(smem_addr(&tfull[acc]), 1));
+          if (lane == 0) {
+            mbar_arrive(&tfull[acc]);
+            if constexpr (PAIR) mbar_arrive_cluster(cluster_map(smem_addr(&tfull[acc]), 1));
+          }
           continue;
         }
         const int kb0 = kSplit ? (t / mn_tiles) * nk / ks : 0, kb1 = kSplit ? (t / mn_tiles + 1) * nk / ks : nk;
         for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&full[stage], phase)) {
+          if (!mbar_wait_warp(&full[stage], phase)) {
             ok = false;
             break;
           }
@@ -422,7 +425,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
             // one K=16 step per k-block: rows of 32 bytes in the 32-byte swizzle,
             // 8-row groups 256 bytes apart
             if constexpr (!PAIR && NB == 1)
-              tc_mma(dtm, sdesc_sw32(a0, 16, 256), sdesc_sw32(b0, 16, 256), idesc, kb != kb0);
+              tc_mma_warp(dtm, sdesc_sw32(a0, 16, 256), sdesc_sw32(b0, 16, 256), idesc, kb != kb0);
           } else {
             // the stage's descriptors once; a K = 16 step is +32 bytes = +2 in
             // the start-address field (the tiles are 1024-byte aligned, so it
@@ -431,19 +434,19 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k) {
               if constexpr (PAIR) {
-                tc_mma_pair(dtm, da + 2 * k, db + 2 * k, idesc, kb != kb0 || k != 0);
+                tc_mma_pair_warp(dtm, da + 2 * k, db + 2 * k, idesc, kb != kb0 || k != 0);
               } else {
-                tc_mma(dtm, da + 2 * k, db + 2 * k, idesc, kb != kb0 || k != 0);
+                tc_mma_warp(dtm, da + 2 * k, db + 2 * k, idesc, kb != kb0 || k != 0);
                 if constexpr (NB == 2)  // low half of the weights: acc += A . W_lo^T
-                  tc_mma(dtm, da + 2 * k, sdesc_sw128(b0 + BSTG / 2, 16, 1024) + 2 * k, idesc, 1u);
+                  tc_mma_warp(dtm, da + 2 * k, sdesc_sw128(b0 + BSTG / 2, 16, 1024) + 2 * k, idesc, 1u);
               }
             }
           }
           issued = true;
           if constexpr (PAIR)
-            tc_commit_pair_multicast(&empty[stage], 0x3);
+            tc_commit_pair_multicast_warp(&empty[stage], 0x3);
           else
-            tc_commit(&empty[stage]);
+            tc_commit_warp(&empty[stage]);
           if (++stage == S) {
             stage = 0;
             phase ^= 1;
@@ -451,19 +454,20 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
         if (ok) {
           if constexpr (PAIR)
-            tc_commit_pair_multicast(&tfull[acc], 0x3);
+            tc_commit_pair_multicast_warp(&tfull[acc], 0x3);
           else
-            tc_commit(&tfull[acc]);
+            tc_commit_warp(&tfull[acc]);
         }
       }
-      if (!ok) record_status(args.status, ELASTO_ERR_TIMEOUT);
+      if (!ok && lane == 0) record_status(args.status, ELASTO_ERR_TIMEOUT);
       // All MMAs this thread issued have finished once `drain` completes.
       if (issued) {
-        if constexpr (PAIR)
-          tc_commit_pair(drain);
-        else
-          tc_commit(drain);
-        mbar_wait(drain, 0);
+        if constexpr (PAIR) {
+          if (elect_one()) tc_commit_pair(drain);
+        } else {
+          tc_commit_warp(drain);
+        }
+        mbar_wait_warp(drain, 0);
       }
     }
   } else if constexpr (TR::tma) {
@@ -490,7 +494,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     volatile uint32_t* fail = tmem_slot + 1 + g;
     uint64_t* rf = rfull + ew * MAX_CBUFS;
     float* sb = sbias + 32 * ew;
-    ChunkIter pf;  // residual prefetch (lane 0)
+    ChunkIter pf;  // residual prefetch (the elected thread)
     long loads = 0, consumed = 0;
     auto fetch = [&](int e) {
       mbar_expect_tx(&rf[e], WBUF);
@@ -499,7 +503,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
       ++loads;
     };
     if constexpr (TR::resid) {
-      if (lane == 0) {
+      if (elect_one()) {
         pf.init(tiles, t_start, t_stride, g, cols);
         for (int e = 0; e < E && pf.valid; ++e) fetch(e);
       }
@@ -571,7 +575,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
           ++consumed;
         } else {
           // the piece is free once the store that last read it (E chunks ago) has done so
-          if (lane == 0) E == 1 ? bulk_wait_read<0>() : bulk_wait_read<1>();
+          if (elect_one()) E == 1 ? bulk_wait_read<0>() : bulk_wait_read<1>();
           if (args.conv)
             named_bar_sync(1 + g, 128);  // (one warp issues the group's stores)
           else
@@ -630,13 +634,12 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
         fence_async_smem();  // (the barriers below also order this chunk's bias reads before the next one's write)
         if (args.conv) {
-          const bool first = q == 0 && lane == 0;  // (its piece is the chunk's first)
           named_bar_sync(1 + g, 128);
           if (*fail) {
             ok = false;
             break;
           }
-          if (first) {
+          if (q == 0 && elect_one()) {  // (its piece is the chunk's first)
             int cb0, cy0, cx0;
             conv_tile(args, m_tile(args, t / nt, mt) * (1 + PAIR) + rank, cb0, cy0, cx0);
             if (cb0 < args.cv_batch) tma_store_4d(&tmC, piece(e), col, cx0, cy0, cb0);  // (a pair's last block may be none)
@@ -644,7 +647,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
           }
         } else {
           __syncwarp();
-          if (lane == 0) {
+          if (elect_one()) {
             if constexpr (TR::resid)
               if (E > 1) bulk_wait_read<0>();  // the previous chunk's store: its piece is refilled below
             if (m0 + q * 32 < M) {
@@ -666,7 +669,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
         }
       }
     }
-    if (lane == 0) {
+    if (elect_one()) {
       if (!ok) record_status(args.status, ELASTO_ERR_TIMEOUT);
       bulk_wait_all();
       // Residual loads issued for chunks never consumed (only on the abort
