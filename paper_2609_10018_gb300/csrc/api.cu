@@ -53,6 +53,7 @@ cudaError_t ensure_kernel_attributes() {
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
   std::call_once(g_attr_once[dev], [dev] {
     cudaError_t r = gemm_init_attributes();
+    if (r == cudaSuccess) r = halo_init_attributes();
     if (r == cudaSuccess) r = attn_init_attributes();
     if (r == cudaSuccess) r = cnn_init_attributes();
     if (r == cudaSuccess) r = pk_init_attributes();

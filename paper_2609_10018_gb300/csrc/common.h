@@ -130,6 +130,20 @@ struct GemmArgs {
   long long split_stride;                    // elements between the partial sums of two splits
 };
 
+// A stride-1 convolution on shared halo tiles (conv.cu).
+struct HaloArgs {
+  int batch, N, bn;             // images (set at launch), output channels, N tile (multiple of 16, <= 256)
+  int Ho, Wo, bw, bh, nbx, nby; // output size, pixel block of a CTA (bw x bh), blocks across and down an image
+  int wp;                       // halo width: pixels between two halo rows in shared memory
+  int taps_x, taps_y, cgroups, pad;
+  int a_tx, a_stage, a_stages;  // bytes of a halo load and of its ring stage, stages
+  int b_stages, b_resident;     // filter ring depth, or the whole filter kept in shared memory
+  const float* bias;
+  void* out;  // f16 [batch, Ho, Wo, ldo]
+  int ldo;
+  int* status;
+};
+
 struct GemmPlan {
   CUtensorMap tmA, tmB, tmB2;  // tmB2: low bf16 plane of W (b_planes == 2)
   CUtensorMap tmC;        // output [M_cap, ldo] (bf16 or fp32), box 128 B x 32 rows, 128B swizzle
@@ -137,6 +151,8 @@ struct GemmPlan {
   GemmArgs args;          // M here is the capacity the A map was encoded for
   int epi = 0;
   bool valid = false;
+  bool use_halo = false;  // a convolution that runs as conv_halo_kernel (halo; tmA and tmB are its maps)
+  HaloArgs halo{};
   // split-K residual plan (gemm_plan_split_resid): after the kernel,
   // rout[r, c] += rbias[c] + sum over splits of the partials, in split order
   const float* rbias = nullptr;
@@ -226,6 +242,16 @@ elasto_status gemm_plan_conv_rows(GemmPlan* p, const void* x, int B_cap, int Hp,
 // Launch for the first M (<= M_cap) rows.
 cudaError_t gemm_launch(const GemmPlan& p, int M, cudaStream_t s);
 cudaError_t gemm_init_attributes();
+// The convolution on halo tiles (conv.cu). halo_layout picks its blocks and
+// shared-memory layout and estimates its nanoseconds; false if the shape does
+// not fit it (N % 8 != 0, a single tap, no room). halo_maps encodes the maps
+// of a plan whose `halo` is filled; x is {channels, x, y, image} = xd with byte
+// strides xs.
+bool halo_layout(HaloArgs* a, int batch, int Ho, int Wo, int taps_x, int taps_y, int cgroups, int pad, int N, int sms,
+                 double* cost);
+bool halo_maps(GemmPlan* p, const void* x, const uint64_t xd[4], const uint64_t xs[3], const void* Wt);
+cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s);
+cudaError_t halo_init_attributes();
 
 // ---------------------------------------------------------------- attention
 struct AttnPlan {

@@ -1,0 +1,482 @@
+// Stride-1 convolution whose input tile is loaded once and read by every tap
+// (Eq. 7's 3x3 convolutions over the kept channels, and the CNN stem).
+//
+// The implicit GEMM of gemm.cu loads one 4-D box per (tap, 64-channel group):
+// a 3x3 convolution brings each input pixel into shared memory nine times, and
+// the boxes, not the tensor cores, set its pace. Here a CTA loads the (bh + taps_y - 1) x
+// (bw + taps_x - 1) halo of its bw x bh output pixels once per channel group.
+// In shared memory a pixel is one 128-byte row, pixels in row-major order of
+// the halo, wp to a row; the accumulator's row r = y * wp + x is output pixel
+// (y, x) of the block, so tap (ky, kx) reads the 128 consecutive halo rows that
+// start at ky * wp + kx: the same tile, another start address (the 128-byte
+// swizzle follows address bits, so a window may start at any row). Rows with
+// x >= bw, and those past the block, compute values that are never stored.
+//
+// Two CTAs on neighbouring SMs work as a pair (tcgen05.mma.cta_group::2,
+// M = 256): each has its own block and half of the filter rows, which halves
+// the filter traffic; all of the filter stays in shared memory where it fits.
+//
+// Roles: warp 0 input producer (and the resident filter), warp 1 MMA issuer
+// (even CTA), warps 2-9 epilogue (two groups of four, every second 64-column
+// chunk each: bias, ReLU, f16, staged through 4 KB of shared memory per warp
+// into 16-byte stores of whole pixels), warp 10 filter producer. Every mbarrier
+// wait is bounded; a timeout records ELASTO_ERR_TIMEOUT.
+//
+// What bounds it: the tensor core takes 64 clocks for a 128-row K = 16 step of
+// up to 128 channels (its input rows arrive at 64 B a clock), so 64 channels
+// run at half the rate of 128. Back-to-back calls, box per tap -> here: 128
+// images of 56 x 56 x 64 -> 64 channels 67.5 -> 35.9 us (62 clocks a step
+// inside), 28 x 28 x 128 -> 128 35.3 -> 20.3 us (1.46 PFLOP/s), 14 x 14 x 192 ->
+// 192 20.6 -> 17.0 us, 16 images of 56 x 56 x 64 12.2 -> 8.4 us. 7 x 7 images
+// (49 of 128 rows) and at most 16 channels stay with the box per tap.
+#include <algorithm>
+
+#include "common.h"
+#include "ptx.cuh"
+
+namespace elasto {
+
+namespace {
+
+constexpr int ROWS = 128;               // accumulator rows of a CTA
+constexpr int EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS + 32;
+constexpr int WBUF = 32 * 128;          // staging of one epilogue warp
+constexpr int POOL = 224 * 1024;        // input stages, filter, staging
+constexpr int MAX_A = 8, MAX_B = 8;     // ring depths
+constexpr int TMEM_COLS = 512, ACC_COLS = 256;
+constexpr size_t SMEM_BYTES = 1024 + POOL + 2048;
+constexpr int BARS = 2 * MAX_A + 2 * MAX_B + 6;  // mbarriers: rings, tfull, tempty, drain, one to pad
+static_assert(BARS * 8 % 16 == 0 && BARS * 8 + EPI_WARPS * 128 + 4 <= 2048, "barriers and bias");
+static_assert(SMEM_BYTES <= 232448, "shared memory");
+
+struct Block {
+  int b, oy, ox;  // image, first output row and column
+};
+__device__ __forceinline__ Block block_at(const HaloArgs& a, int i) {
+  const int r = i / a.nbx;
+  return {r / a.nby, (r % a.nby) * a.bh, (i - r * a.nbx) * a.bw};
+}
+
+template <bool RELU>
+__global__ void __launch_bounds__(THREADS, 1)
+    conv_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+                     const HaloArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int taps = a.taps_x * a.taps_y, nk = taps * a.cgroups;
+  const int half = a.bn / 2;            // filter rows of one CTA's k-block
+  const int b_bytes = half * 128;
+  uint8_t* sA = smem;
+  uint8_t* sB = sA + a.a_stages * a.a_stage;
+  uint8_t* sC = smem + POOL - EPI_WARPS * WBUF;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + POOL);
+  uint64_t* a_full = bars;
+  uint64_t* a_empty = a_full + MAX_A;
+  uint64_t* b_full = a_empty + MAX_A;  // (resident filter: b_full[0])
+  uint64_t* b_empty = b_full + MAX_B;
+  uint64_t* tfull = b_empty + MAX_B;
+  uint64_t* tempty = tfull + 2;
+  uint64_t* drain = tempty + 2;
+  float* sbias = reinterpret_cast<float*>(bars + BARS);  // 32 values per epilogue warp, read as float4
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sbias + 32 * EPI_WARPS);
+
+  const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int blocks = a.batch * a.nby * a.nbx;
+  const int nt = (a.N + a.bn - 1) / a.bn;
+  const int tiles = (blocks + 1) / 2 * nt;
+  const int rank = warp_uniform(static_cast<int>(cluster_ctarank()));
+  const bool leader = rank == 0;
+  const int t0 = warp_uniform(static_cast<int>(cluster_id_x()));
+  const int step = warp_uniform(static_cast<int>(cluster_count_x()));
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < MAX_A; ++s) {
+      mbar_init(&a_full[s], 1);
+      mbar_init(&a_empty[s], 1);
+    }
+    for (int s = 0; s < MAX_B; ++s) {
+      mbar_init(&b_full[s], 1);
+      mbar_init(&b_empty[s], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&tfull[i], 1);
+      mbar_init(&tempty[i], 2 * EPI_WARPS);
+    }
+    mbar_init(drain, 1);
+    fence_barrier_init();
+  }
+  if (warp == 0) {
+    tmem_alloc_pair(tmem_slot, TMEM_COLS);
+    tmem_relinquish_pair();
+  }
+  if (warp == 1 && elect_one()) {
+    tma_prefetch_desc(&tmX);
+    tma_prefetch_desc(&tmW);
+  }
+  tc_fence_before();
+  cluster_sync_all();  // both CTAs' barriers initialised before any remote arrive
+  tc_fence_after();
+  const uint32_t tmem = warp_uniform(static_cast<int>(*tmem_slot));
+  // The filter is not written by an earlier kernel of a stream that triggers
+  // early: its producers start before the wait for that kernel.
+  if (a.b_resident && warp == 0 && t0 < tiles && elect_one()) {
+    if (leader) mbar_expect_tx(&b_full[0], 2u * nk * b_bytes);
+    const uint32_t bar = cluster_map(smem_addr(&b_full[0]), 0);
+    for (int k = 0; k < nk; ++k) tma_load_2d_pair(sB + k * b_bytes, &tmW, bar, k * 64, rank * half);
+  }
+  if (warp != 10 || a.b_resident) {
+    pdl_wait();
+    pdl_trigger();
+  }
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ input producer
+    if (elect_one()) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      long issued = 0;
+      for (int t = t0; t < tiles && ok; t += step) {
+        // (the last pair's second block may not exist: b = batch, all read as zero or never stored)
+        const Block k = block_at(a, (t / nt) * 2 + rank);
+        for (int g = 0; g < a.cgroups; ++g) {
+          if (!mbar_wait(&a_empty[s], ph ^ 1)) {
+            ok = false;
+            break;
+          }
+          if (leader) mbar_expect_tx(&a_full[s], 2u * a.a_tx);
+          tma_load_4d_pair(sA + s * a.a_stage, &tmX, cluster_map(smem_addr(&a_full[s]), 0), g * 64, k.ox - a.pad,
+                           k.oy - a.pad, k.b);
+          ++issued;
+          if (++s == a.a_stages) {
+            s = 0;
+            ph ^= 1;
+          }
+        }
+      }
+      if (!ok) record_status(a.status, ELASTO_ERR_TIMEOUT);
+      // no copy may still be landing when the CTAs exit: the even CTA's
+      // barriers count both CTAs' bytes, and the cluster barrier below keeps
+      // the odd CTA until they are in
+      for (long i = issued > a.a_stages ? issued - a.a_stages : 0; leader && i < issued; ++i)
+        mbar_wait(&a_full[i % a.a_stages], static_cast<uint32_t>((i / a.a_stages) & 1));
+      if (leader && a.b_resident && t0 < tiles) mbar_wait(&b_full[0], 0);
+    }
+  } else if (warp == 10) {
+    // ------------------------------------------------------------ filter producer
+    if (!a.b_resident && elect_one()) {
+      int s = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      long issued = 0;
+      for (int t = t0; t < tiles && ok; t += step) {
+        const int row = (t % nt) * a.bn + rank * half;
+        for (int g = 0; g < a.cgroups && ok; ++g)
+          for (int tap = 0; tap < taps; ++tap) {
+            if (!mbar_wait(&b_empty[s], ph ^ 1)) {
+              ok = false;
+              break;
+            }
+            if (leader) mbar_expect_tx(&b_full[s], 2u * b_bytes);
+            tma_load_2d_pair(sB + s * b_bytes, &tmW, cluster_map(smem_addr(&b_full[s]), 0),
+                             (tap * a.cgroups + g) * 64, row);
+            ++issued;
+            if (++s == a.b_stages) {
+              s = 0;
+              ph ^= 1;
+            }
+          }
+      }
+      if (!ok) record_status(a.status, ELASTO_ERR_TIMEOUT);
+      for (long i = issued > a.b_stages ? issued - a.b_stages : 0; leader && i < issued; ++i)
+        mbar_wait(&b_full[i % a.b_stages], static_cast<uint32_t>((i / a.b_stages) & 1));
+    }
+    if (!a.b_resident) {
+      pdl_wait();
+      pdl_trigger();
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer
+    if (leader) {
+      const uint32_t idesc = idesc_16_f32(2 * ROWS, a.bn, true);
+      int as = 0, bs = 0, local = 0;
+      uint32_t aph = 0, bph = 0;
+      bool ok = t0 >= tiles || !a.b_resident || mbar_wait_warp(&b_full[0], 0);
+      bool issued = false;
+      for (int t = t0; t < tiles && ok; t += step, ++local) {
+        const int acc = local & 1;
+        if (!mbar_wait_warp(&tempty[acc], static_cast<uint32_t>((local >> 1) & 1) ^ 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + acc * ACC_COLS;
+        for (int g = 0; g < a.cgroups && ok; ++g) {
+          if (!mbar_wait_warp(&a_full[as], aph)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          uint64_t row = sdesc_sw128(smem_addr(sA + as * a.a_stage), 16, 1024);  // tap (ky, 0): +8 per halo row
+          int tap = 0;
+          for (int ky = 0; ky < a.taps_y && ok; ++ky, row += 8 * a.wp)
+            for (int kx = 0; kx < a.taps_x; ++kx, ++tap) {
+              if (!a.b_resident) {
+                if (!mbar_wait_warp(&b_full[bs], bph)) {
+                  ok = false;
+                  break;
+                }
+                tc_fence_after();
+              }
+              const uint64_t da = row + 8 * kx;
+              const uint64_t db =
+                  sdesc_sw128(smem_addr(sB + (a.b_resident ? tap * a.cgroups + g : bs) * b_bytes), 16, 1024);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) tc_mma_pair_warp(d, da + 2 * k, db + 2 * k, idesc, (g | tap | k) != 0);
+              issued = true;
+              if (!a.b_resident) {
+                tc_commit_pair_multicast_warp(&b_empty[bs], 0x3);
+                if (++bs == a.b_stages) {
+                  bs = 0;
+                  bph ^= 1;
+                }
+              }
+            }
+          tc_commit_pair_multicast_warp(&a_empty[as], 0x3);
+          if (++as == a.a_stages) {
+            as = 0;
+            aph ^= 1;
+          }
+        }
+        if (ok) tc_commit_pair_multicast_warp(&tfull[acc], 0x3);
+      }
+      if (!ok && lane == 0) record_status(a.status, ELASTO_ERR_TIMEOUT);
+      if (issued) {  // every MMA has finished once `drain` completes
+        if (elect_one()) tc_commit_pair(drain);
+        mbar_wait_warp(drain, 0);
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int ew = warp - 2, q = warp & 3, grp = ew >> 2;
+    uint8_t* buf = sC + ew * WBUF;
+    float* sb = sbias + 32 * ew;
+    // this lane's part of the stores: 16 bytes (8 channels) of eight pixels
+    const int piece = lane & 7;
+    int rel[8], pos[8];  // pixel offset from the block's first, (y << 16 | x); pos < 0: not an output
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int r = q * 32 + i * 4 + (lane >> 3), y = r / a.wp, x = r - y * a.wp;
+      rel[i] = y * a.Wo + x;
+      pos[i] = y < a.bh && x < a.bw ? (y << 16 | x) : -1;
+    }
+    const uint32_t row_tm = tmem + (static_cast<uint32_t>(q * 32) << 16);
+    int local = 0, before = 0;
+    bool ok = true;
+    for (int t = t0; t < tiles; t += step, ++local) {
+      const int acc = local & 1, bi = (t / nt) * 2 + rank, n0 = (t % nt) * a.bn;
+      const int width = min(a.bn, a.N - n0), chunks = (width + 63) / 64;
+      int c = grp ^ before;
+      before ^= chunks & 1;
+      float nb[2];
+      auto bias_of = [&](int chunk) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int k = chunk * 64 + 32 * h + lane;
+          nb[h] = a.bias && k < width ? __ldg(a.bias + n0 + k) : 0.0f;
+        }
+      };
+      bias_of(c);
+      ok = __all_sync(0xffffffffu, mbar_wait(&tfull[acc], static_cast<uint32_t>((local >> 1) & 1)));
+      if (!ok) break;
+      tc_fence_after();
+      auto release = [&] {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(cluster_map(smem_addr(&tempty[acc]), 0));
+      };
+      if (c >= chunks) release();
+      const Block k = block_at(a, bi);
+      for (; c < chunks; c += 2) {
+        uint32_t v[2][32];
+        tmem_ld_32x32b_x32(row_tm + acc * ACC_COLS + c * 64, v[0]);
+        tmem_ld_32x32b_x32(row_tm + acc * ACC_COLS + c * 64 + 32, v[1]);
+        const float bl[2] = {nb[0], nb[1]};
+        if (c + 2 < chunks) bias_of(c + 2);
+        tmem_ld_wait();
+        if (c + 2 >= chunks) release();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          __syncwarp();
+          sb[lane] = bl[h];
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t ow[4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const float4 b4 = reinterpret_cast<const float4*>(sb)[2 * j + i];
+              float2 lo = add2(make_float2(__uint_as_float(v[h][8 * j + 4 * i]), __uint_as_float(v[h][8 * j + 4 * i + 1])),
+                               make_float2(b4.x, b4.y));
+              float2 hi =
+                  add2(make_float2(__uint_as_float(v[h][8 * j + 4 * i + 2]), __uint_as_float(v[h][8 * j + 4 * i + 3])),
+                       make_float2(b4.z, b4.w));
+              if (RELU) {
+                lo = make_float2(fmaxf(lo.x, 0.0f), fmaxf(lo.y, 0.0f));
+                hi = make_float2(fmaxf(hi.x, 0.0f), fmaxf(hi.y, 0.0f));
+              }
+              ow[2 * i] = pack_f16x2(lo.x, lo.y);
+              ow[2 * i + 1] = pack_f16x2(hi.x, hi.y);
+            }
+            *reinterpret_cast<uint4*>(buf + lane * 128 + (((4 * h + j) ^ (lane & 7)) << 4)) =
+                make_uint4(ow[0], ow[1], ow[2], ow[3]);
+          }
+        }
+        __syncwarp();
+        const int col = c * 64 + piece * 8;
+        if (bi < blocks && col < width) {
+          uint4* dst = reinterpret_cast<uint4*>(static_cast<__half*>(a.out) +
+                                                ((static_cast<size_t>(k.b) * a.Ho + k.oy) * a.Wo + k.ox) * a.ldo + n0 +
+                                                col);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int r = i * 4 + (lane >> 3);
+            if (pos[i] >= 0 && k.oy + (pos[i] >> 16) < a.Ho && k.ox + (pos[i] & 0xffff) < a.Wo)
+              dst[static_cast<size_t>(rel[i]) * a.ldo / 8] =
+                  *reinterpret_cast<const uint4*>(buf + r * 128 + ((piece ^ (r & 7)) << 4));
+          }
+        }
+        __syncwarp();  // the staging rows are read before the next chunk writes them
+      }
+    }
+    if (!ok && lane == 0) record_status(a.status, ELASTO_ERR_TIMEOUT);
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // the peer's TMEM, barriers and copies are no longer in use
+  if (warp == 0) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, TMEM_COLS);
+  }
+}
+
+int round_up(int v, int m) { return (v + m - 1) / m * m; }
+
+}  // namespace
+
+cudaError_t halo_init_attributes() {
+  const int bytes = static_cast<int>(SMEM_BYTES);
+  cudaError_t e = cudaFuncSetAttribute(conv_halo_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(conv_halo_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+bool halo_layout(HaloArgs* a, int batch, int Ho, int Wo, int taps_x, int taps_y, int cgroups, int pad, int N, int sms,
+                 double* cost) {
+  if (taps_x * taps_y < 2 || N % 8 != 0) return false;
+  *a = HaloArgs{};
+  a->batch = batch;
+  a->Ho = Ho;
+  a->Wo = Wo;
+  a->N = N;
+  a->taps_x = taps_x;
+  a->taps_y = taps_y;
+  a->cgroups = cgroups;
+  a->pad = pad;
+  // output block: the fewest blocks per image whose last pixel's row still
+  // fits the 128 accumulator rows, then the smallest halo
+  long best_blocks = -1;
+  int best_rows = 0;
+  for (int bw = 1; bw <= Wo && bw <= ROWS; ++bw) {
+    const int wp = bw + taps_x - 1, bh = std::min(Ho, (ROWS - bw) / wp + 1);
+    const int nbx = (Wo + bw - 1) / bw, nby = (Ho + bh - 1) / bh;
+    const int bh_even = (Ho + nby - 1) / nby;  // the same number of blocks, evenly high
+    const int rows = wp * (bh_even + taps_y - 1);
+    if (wp > 256 || bh_even + taps_y - 1 > 256) continue;
+    const long n = static_cast<long>(nbx) * nby;
+    if (best_blocks < 0 || n < best_blocks || (n == best_blocks && rows < best_rows)) {
+      best_blocks = n;
+      best_rows = rows;
+      a->bw = bw;
+      a->bh = bh_even;
+      a->nbx = nbx;
+      a->nby = nby;
+      a->wp = wp;
+    }
+  }
+  if (best_blocks < 0) return false;
+  a->a_tx = best_rows * 128;
+  a->a_stage = round_up(a->a_tx, 1024);
+  // the last tap's window ends this many rows past the halo's end: the rows
+  // read there (never used) have to be shared memory too
+  const int over = (ROWS + (taps_y - 1) * a->wp + taps_x - 1 - best_rows) * 128;
+  const int pool = POOL - EPI_WARPS * WBUF, nk = taps_x * taps_y * cgroups;
+  if (over > EPI_WARPS * WBUF) return false;
+  const int units = sms / 2;
+  *cost = -1.0;
+  HaloArgs pick = *a;
+  for (int n_tiles = (N + 255) / 256; n_tiles <= (N + 15) / 16; n_tiles *= 2) {
+    HaloArgs b = *a;
+    b.bn = round_up((N + n_tiles - 1) / n_tiles, 16);
+    const int nt = (N + b.bn - 1) / b.bn, b_bytes = b.bn / 2 * 128;
+    b.b_resident = nt == 1 && 2 * b.a_stage + nk * b_bytes <= pool ? 1 : 0;
+    if (b.b_resident) {
+      b.a_stages = std::min((pool - nk * b_bytes) / b.a_stage, MAX_A);
+      b.b_stages = 1;
+    } else {
+      // two input stages (three where that leaves the filter ring full), the rest filter
+      b.a_stages = cgroups > 1 && pool - 3 * b.a_stage >= MAX_B * b_bytes ? 3 : 2;
+      b.b_stages = std::min((pool - b.a_stages * b.a_stage) / b_bytes, MAX_B);
+      if (pool < b.a_stages * b.a_stage || b.b_stages < 3) continue;
+    }
+    // a 128-row K = 16 step takes 64 clocks up to 128 channels; a filter wait per k-block adds ~130
+    const double mma = (4 * std::max(0.5 * b.bn, 64.0) + (b.b_resident ? 0 : 130)) / 1.9;
+    const double load = (b.a_tx / (taps_x * taps_y) + (b.b_resident ? 0 : b_bytes)) / 126.0;
+    const long tiles = (best_blocks * batch + 1) / 2 * nt, waves = (tiles + units - 1) / units;
+    const double epilogue = 500.0 + 6.0 * b.bn;
+    const double c = waves * (std::max(nk * std::max(mma, load), epilogue) + 150.0) + epilogue + 1000.0;
+    if (*cost < 0 || c < *cost) {
+      *cost = c;
+      pick = b;
+    }
+    if (b.bn <= 64) break;
+  }
+  if (*cost < 0) return false;
+  *a = pick;
+  return true;
+}
+
+bool halo_maps(GemmPlan* p, const void* x, const uint64_t xd[4], const uint64_t xs[3], const void* Wt) {
+  const HaloArgs& a = p->halo;
+  const uint32_t box[4] = {64u, static_cast<uint32_t>(a.wp), static_cast<uint32_t>(a.bh + a.taps_y - 1), 1u};
+  const uint32_t es[4] = {1u, 1u, 1u, 1u};
+  const uint64_t K = static_cast<uint64_t>(a.taps_x) * a.taps_y * a.cgroups * 64;
+  return encode_tmap_4d(&p->tmA, x, xd, xs, box, es, false) &&
+         encode_tmap_2d(&p->tmB, Wt, K, a.N, K * 2, 64, a.bn / 2);
+}
+
+cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s) {
+  HaloArgs a = p.halo;
+  a.batch = batch;
+  const int nt = (a.N + a.bn - 1) / a.bn, blocks = batch * a.nby * a.nbx;
+  const int clusters = std::min((blocks + 1) / 2 * nt, num_sms() / 2);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(2 * clusters);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return p.epi == EPI_BIAS_RELU_F16 ? cudaLaunchKernelEx(&cfg, conv_halo_kernel<true>, p.tmA, p.tmB, a)
+                                    : cudaLaunchKernelEx(&cfg, conv_halo_kernel<false>, p.tmA, p.tmB, a);
+}
+
+}  // namespace elasto

@@ -1167,6 +1167,24 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
   a.b_resident = (N <= a.bn && 4 * A_STAGE + b_all + CBUF <= POOL) ? 1 : 0;
   if (!a.b_resident && !k16) choose_tile(prob, 64, true, &a.bn, &pair);
   a.pair = pair ? 1 : 0;
+  // halo tiles where they are estimated faster than a box per tap
+  double halo = 0.0;
+  if (!k16 && stride == 1 &&
+      halo_layout(&p->halo, B_cap, Ho, Wo, taps_x, taps / taps_x, cg, pad, N, prob.sms, &halo) &&
+      halo < tile_cost(prob, a.bn, pair)) {
+    p->halo.bias = bias;
+    p->halo.out = out;
+    p->halo.ldo = ldo;
+    p->halo.status = status;
+    if (!halo_maps(p, x, xd, xs, Wt)) {
+      set_error(std::string(who) + ": cuTensorMapEncodeTiled failed (alignment or size)");
+      return ELASTO_ERR_UNSUPPORTED;
+    }
+    p->use_halo = true;
+    p->epi = epi;
+    p->valid = true;
+    return ELASTO_OK;
+  }
   a.b_stage = (a.pair ? a.bn / 2 : a.bn) * (a.b_resident ? bke : BK) * 2;
   const int ring = POOL - (a.b_resident ? b_all : 0), stage = A_STAGE + (a.b_resident ? 0 : a.b_stage);
   a.stages = std::min((ring - CBUF) / stage, MAX_STAGES);
@@ -1313,6 +1331,7 @@ cudaError_t gemm_launch_main(const GemmPlan& p, int M, cudaStream_t s) {
 
 cudaError_t gemm_launch(const GemmPlan& p, int M, cudaStream_t s) {
   if (M <= 0) return cudaSuccess;
+  if (p.use_halo) return halo_launch(p, M, s);
   if (p.args.ksplit <= 1) return gemm_launch_main(p, M, s);
   if (M > p.rcap) return cudaErrorInvalidValue;  // the partial buffer holds rcap rows
   cudaError_t e = gemm_launch_main(p, M, s);
