@@ -9,30 +9,36 @@
 // heads concatenated in the same order (the K axis of the packed W^O).
 //
 // Persistent kernel; a work item is one (image, kept head) and needs at most
-// two 128-query tiles (n <= 256). Items run from the last image to the first:
-// the QKV GEMM wrote its rows in increasing order, so the most recent (still
-// in L2) are read first. Roles:
+// two 128-query tiles (n <= 256); its unit is one query tile. Items run from
+// the last image to the first: the QKV GEMM wrote its rows in increasing order,
+// so the most recent (still in L2) are read first. Roles:
 //   warp 0      TMA producer: K and V of an item into one of `kv_slots`
 //               shared-memory slots, its query tiles into one of two Q
 //               buffers per tile (3-D maps: rows past n read as zero);
-//   warp 1      tcgen05.mma issuer: S_t = Q_t K^T (M=128, N=n_pad, K=64) into
-//               the 256-column TMEM region of query tile t, then O_t = P_t V
-//               with P_t read from TMEM (M=128, N=64, K=n_pad; V MN-major);
-//   warps 2-9   two groups of four, one per query tile: one query row per
-//               thread (TMEM lane = row). Row max and exp2 numerators over the
-//               n valid keys in fp32; P_t stored back into TMEM as bf16 pairs
-//               over the S columns already consumed; then O row * (1 / row
-//               sum) -> bf16, 128 contiguous bytes per thread. Warps whose 32
-//               rows are all padding (past n) skip the TMEM work.
-// The two query tiles run half an item apart: the issue order is
-//   S(0,0); then per item k: S(k,1), PV(k,0), S(k+1,0), PV(k,1)
-// so the tensor pipe computes one tile's MMAs while the other tile's group
-// runs its softmax (both softmaxes at once would share the exp units while
-// the tensor pipe idles). An item's K/V slot is released after PV(k,1), its
-// Q buffers after S(k,1).
-// TMEM per tile region: S in [0, n_pad), P in [0, n_pad / 2), O in [128, 192)
-// (O overwrites S columns the softmax has consumed, so S(k+1,t) waits until
-// O(k,t) is read out).
+//   warp 1      tcgen05.mma issuer: S = Q K^T (M=128, N=n_pad, K=64) into the
+//               256-column TMEM region of the unit's group, then O = P V with P
+//               read from TMEM (M=128, N=64, K=n_pad; V MN-major);
+//   warps 2-9   two groups of four, which take the units in turn: one query
+//               row per thread (TMEM lane = row). Row max and exp2 numerators
+//               over the n valid keys in fp32 (softmax_row); P stored back into
+//               TMEM as bf16 pairs over the S columns already consumed; then
+//               O row * (1 / row sum) -> bf16, staged in shared memory and
+//               stored by 32-row TMA boxes (rows past n are clipped). Warps
+//               whose 32 rows are all padding skip the TMEM work.
+// The issue order is S(0); then per unit u: S(u+1), PV(u), so the tensor pipe
+// computes one group's MMAs while the other runs its softmax. An item's K/V
+// slot is released after its last PV, its Q buffers after its last S.
+// TMEM per group: S in [0, n_pad), P in [0, n_pad / 2), O in [128, 192) (O
+// overwrites S columns the softmax has consumed, so a group's next S waits
+// until its O is read out).
+// What bounds it: each unit is a serial chain S -> softmax -> PV -> read-out and
+// TMEM holds two. ViT-B (256 images, 197 tokens, 12 heads), per unit: softmax
+// 2300 clocks (1660 of them the exponentials), PV 1000-1400, scaling and staging
+// O 900, S 300; 86.7 -> 61.9 us a call, the memory's share being 46. Before, the
+// softmax took 3700 (packed arithmetic and pipelined reads since) and storing
+// 16 bytes to each of 32 rows per instruction 1500-2000 (TMA boxes since). With
+// one query tile per item the second group had no work: 128 tokens 51.5 -> 34.3
+// us, 65 tokens x 3 heads 13.7 -> 7.8.
 // Scale 1/sqrt(64) (the base model's head width; it does not change with the
 // number of kept heads). Every mbarrier wait is bounded.
 #include "common.h"
@@ -48,18 +54,20 @@ constexpr int QT = 128;                     // queries per tile
 constexpr int MAXK = 256;                   // max keys
 constexpr int Q_BYTES = QT * HD * 2;        // 16 KB
 constexpr int QBUF_BYTES = 4 * Q_BYTES;     // two buffers per query tile
+constexpr int O_BYTES = 32 * HD * 2;        // output staging of one softmax warp
+constexpr int OBUF_BYTES = 8 * O_BYTES;
 constexpr int BAR_BYTES = 256;
 constexpr int SMEM_LIMIT = 232448;          // dynamic shared memory per block on sm_103
 constexpr int TMEM_COLS = 512;
 constexpr int O_COL = 128;
 
-// Shared memory: [Q buffers][KV slots][barriers], 1024-byte aligned.
+// Shared memory: [Q buffers][output staging][KV slots][barriers], 1024-byte aligned.
 __host__ __device__ constexpr int kv_slot_bytes(int n_pad) { return 2 * n_pad * HD * 2; }
 __host__ __device__ constexpr int kv_slots_for(int n_pad) {
-  return 1024 + QBUF_BYTES + 3 * kv_slot_bytes(n_pad) + BAR_BYTES <= SMEM_LIMIT ? 3 : 2;
+  return 1024 + QBUF_BYTES + OBUF_BYTES + 3 * kv_slot_bytes(n_pad) + BAR_BYTES <= SMEM_LIMIT ? 3 : 2;
 }
 __host__ __device__ constexpr int smem_bytes_for(int n_pad) {
-  return 1024 + QBUF_BYTES + kv_slots_for(n_pad) * kv_slot_bytes(n_pad) + BAR_BYTES;
+  return 1024 + QBUF_BYTES + OBUF_BYTES + kv_slots_for(n_pad) * kv_slot_bytes(n_pad) + BAR_BYTES;
 }
 __host__ __device__ constexpr int max_smem_bytes() {
   int m = 0;
@@ -68,32 +76,115 @@ __host__ __device__ constexpr int max_smem_bytes() {
 }
 static_assert(max_smem_bytes() <= SMEM_LIMIT, "attention shared memory");
 
+constexpr float kScale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
+
+__device__ __forceinline__ void load64(uint32_t tm, uint32_t (&v)[2][32]) {
+  tmem_ld_32x32b_x32(tm, v[0]);
+  tmem_ld_32x32b_x32(tm + 32, v[1]);
+}
+
+// Softmax of one score row (this thread's TMEM lane, columns tm .. tm + n):
+// the numerators exp2((s - max) * kScale) go back as bf16 pairs over the
+// columns already consumed, zeros up to the next multiple of 16; returns their
+// fp32 sum. NF = n / 64 whole chunks without masks, then the 1 to 63 columns
+// left in masked pieces of 16.
+//
+// The row is bound by instruction issue and by the TMEM round trips (300 to
+// 600 clocks while MMAs run). So: packed fp32 multiply-adds and sums and
+// three-input maxima (3 issue slots a score instead of 4.5); nothing read past
+// the last piece (n = 197: 208 columns instead of 256, most of the last 64
+// masked); each chunk in flight while the one before it is worked on.
+template <int NF>
+__device__ __forceinline__ float softmax_row(uint32_t tm, int n) {
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+  uint32_t v[2][2][32];
+  if constexpr (NF > 0) load64(tm, v[0]);
+#pragma unroll
+  for (int i = 0; i < NF; ++i) {
+    tmem_ld_wait();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (i + 1 < NF) tmem_ld_32x32b_x32(tm + 64 * (i + 1) + 32 * h, v[(i + 1) & 1][h]);
+#pragma unroll
+      for (int j = 0; j < 32; j += 2)
+        m[(j >> 1) & 3] = max3(m[(j >> 1) & 3], __uint_as_float(v[i & 1][h][j]), __uint_as_float(v[i & 1][h][j + 1]));
+    }
+  }
+  for (int c = 64 * NF; c < n; c += 16) {
+    uint32_t w[16];
+    tmem_ld_16(tm + c, w);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (c + j < n) m[j & 3] = fmaxf(m[j & 3], __uint_as_float(w[j]));
+  }
+  const float neg = -fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])) * kScale;
+  const float2 scale2 = make_float2(kScale, kScale), neg2 = make_float2(neg, neg);
+  float2 s[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+  if constexpr (NF > 0) load64(tm, v[0]);
+#pragma unroll
+  for (int i = 0; i < NF; ++i) {
+    tmem_ld_wait();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (i + 1 < NF) tmem_ld_32x32b_x32(tm + 64 * (i + 1) + 32 * h, v[(i + 1) & 1][h]);
+      uint32_t pk[16];
+#pragma unroll
+      for (int j = 0; j < 32; j += 2) {
+        const float2 x = fma2(make_float2(__uint_as_float(v[i & 1][h][j]), __uint_as_float(v[i & 1][h][j + 1])), scale2,
+                              neg2);
+        const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+        s[(j >> 1) & 3] = add2(s[(j >> 1) & 3], p);
+        pk[j >> 1] = pack_bf16x2(p.x, p.y);
+      }
+      tmem_st_16(tm + 32 * i + 16 * h, pk);
+    }
+  }
+  for (int c = 64 * NF; c < n; c += 16) {
+    uint32_t w[16], pk[8];
+    tmem_ld_16(tm + c, w);
+    tmem_ld_wait();
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+      const float2 x = fma2(make_float2(__uint_as_float(w[j]), __uint_as_float(w[j + 1])), scale2, neg2);
+      const float2 p = make_float2(c + j < n ? ex2_approx(x.x) : 0.0f, c + j + 1 < n ? ex2_approx(x.y) : 0.0f);
+      s[(j >> 1) & 3] = add2(s[(j >> 1) & 3], p);
+      pk[j >> 1] = pack_bf16x2(p.x, p.y);
+    }
+    tmem_st_8(tm + (c >> 1), pk);
+  }
+  const float2 t = add2(add2(s[0], s[1]), add2(s[2], s[3]));
+  return t.x + t.y;
+}
+
 __global__ void __launch_bounds__(THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
-                   bf16* __restrict__ out, int n, int n_pad, int heads, int items, int blk_stride,
+                   const __grid_constant__ CUtensorMap tmO, int n, int n_pad, int heads, int items, int blk_stride,
                    int head_stride, int* status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int ns = kv_slots_for(n_pad);
   const int slot_bytes = kv_slot_bytes(n_pad);
   uint8_t* qbuf = smem;                                    // [tile][parity] Q_BYTES each
-  uint8_t* kvbuf = smem + QBUF_BYTES;                      // [slot] K then V, n_pad rows of 128 B
+  uint8_t* obuf = smem + QBUF_BYTES;                       // [softmax warp] 32 rows of 128 B
+  uint8_t* kvbuf = obuf + OBUF_BYTES;                      // [slot] K then V, n_pad rows of 128 B
   uint64_t* bars = reinterpret_cast<uint64_t*>(kvbuf + ns * slot_bytes);
   uint64_t* full = bars + 0;        // [3] item k's Q, K, V landed (slot k % ns)
   uint64_t* kv_empty = bars + 3;    // [3] slot's PV MMAs finished
   uint64_t* q_empty = bars + 6;     // [2] Q buffers of parity k & 1 consumed by S(k, *)
-  uint64_t* s_full = bars + 8;      // [2] S_t in TMEM
-  uint64_t* p_full = bars + 10;     // [2] P_t in TMEM (128 arrivals)
-  uint64_t* o_full = bars + 12;     // [2] O_t in TMEM
-  uint64_t* o_empty = bars + 14;    // [2] O_t read out (128 arrivals)
+  uint64_t* s_full = bars + 8;      // [2] the group's S in TMEM
+  uint64_t* p_full = bars + 10;     // [2] its P in TMEM (128 arrivals)
+  uint64_t* o_full = bars + 12;     // [2] its O in TMEM
+  uint64_t* o_empty = bars + 14;    // [2] its O read out (128 arrivals)
   uint64_t* drain = bars + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
 
   const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int w = heads * HD;
   const int tiles = n > QT ? 2 : 1;
   // items of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
   const int nk = items > static_cast<int>(blockIdx.x) ? (items - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  // unit u: query tile u % tiles of item u / tiles, worked on by group u & 1
+  const int units = nk * tiles;
 
   if (threadIdx.x == 0) {
     for (int k = 0; k < 3; ++k) {
@@ -154,42 +245,38 @@ __global__ void __launch_bounds__(THREADS, 1)
       const uint32_t idesc_s = idesc_bf16_f32(QT, n_pad);
       const uint32_t idesc_o = idesc_bf16_f32(QT, HD, false, true);
       bool ok = true;
-      // S(k, t): needs item k landed (waited once, at t = 0) and O(k-1, t)
-      // read out (S overwrites the O columns of its tile region)
-      auto issue_s = [&](int k, int t) -> bool {
-        const int slot = k % ns;
+      // S(u): needs its item landed (waited once, at the first tile) and the
+      // group's previous O read out (S overwrites the O columns)
+      auto issue_s = [&](int u) -> bool {
+        const int k = tiles == 2 ? u >> 1 : u, t = tiles == 2 ? u & 1 : 0, g = u & 1, slot = k % ns;
         if (t == 0 && !mbar_wait_warp(&full[slot], (k / ns) & 1)) return false;
-        if (!mbar_wait_warp(&o_empty[t], (k & 1) ^ 1)) return false;
+        if (!mbar_wait_warp(&o_empty[g], ((u >> 1) & 1) ^ 1)) return false;
         tc_fence_after();
-        const uint32_t q0 = smem_addr(qbuf + (2 * t + (k & 1)) * Q_BYTES);
-        const uint32_t k0 = smem_addr(kvbuf + slot * slot_bytes);
+        const uint64_t dq = sdesc_sw128(smem_addr(qbuf + (2 * t + (k & 1)) * Q_BYTES), 16, 1024);
+        const uint64_t dk = sdesc_sw128(smem_addr(kvbuf + slot * slot_bytes), 16, 1024);
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk)
-          tc_mma_warp(tmem + t * 256, sdesc_sw128(q0 + kk * 32, 16, 1024), sdesc_sw128(k0 + kk * 32, 16, 1024), idesc_s,
-                 kk != 0);
-        tc_commit_warp(&s_full[t]);
+        for (int kk = 0; kk < HD / 16; ++kk) tc_mma_warp(tmem + g * 256, dq + 2 * kk, dk + 2 * kk, idesc_s, kk != 0);
+        tc_commit_warp(&s_full[g]);
         if (t == tiles - 1) tc_commit_warp(&q_empty[k & 1]);
         return true;
       };
-      // PV(k, t): needs P(k, t) in TMEM
-      auto issue_pv = [&](int k, int t) -> bool {
-        if (!mbar_wait_warp(&p_full[t], k & 1)) return false;
+      // PV(u): needs P(u) in TMEM
+      auto issue_pv = [&](int u) -> bool {
+        const int k = tiles == 2 ? u >> 1 : u, t = tiles == 2 ? u & 1 : 0, g = u & 1;
+        if (!mbar_wait_warp(&p_full[g], (u >> 1) & 1)) return false;
         tc_fence_after();
-        const uint32_t v0 = smem_addr(kvbuf + (k % ns) * slot_bytes + slot_bytes / 2);
-        for (int s = 0; s < n_pad / 16; ++s)
-          tc_mma_tmem_a_warp(tmem + t * 256 + O_COL, tmem + t * 256 + 8 * s, sdesc_sw128(v0 + s * 16 * 128, 16384, 1024),
-                        idesc_o, s != 0);
-        tc_commit_warp(&o_full[t]);
+        const uint64_t dv = sdesc_sw128(smem_addr(kvbuf + (k % ns) * slot_bytes + slot_bytes / 2), 16384, 1024);
+        for (int s = 0; s < n_pad / 16; ++s)  // 16 keys are 16 rows of 128 bytes
+          tc_mma_tmem_a_warp(tmem + g * 256 + O_COL, tmem + g * 256 + 8 * s, dv + 128 * s, idesc_o, s != 0);
+        tc_commit_warp(&o_full[g]);
         if (t == tiles - 1) tc_commit_warp(&kv_empty[k % ns]);
         return true;
       };
-      ok = issue_s(0, 0);
+      ok = issue_s(0);
       const bool issued = ok;
-      for (int k = 0; k < nk && ok; ++k) {
-        if (tiles == 2) ok = issue_s(k, 1);
-        if (ok) ok = issue_pv(k, 0);
-        if (ok && k + 1 < nk) ok = issue_s(k + 1, 0);
-        if (ok && tiles == 2) ok = issue_pv(k, 1);
+      for (int u = 0; u < units && ok; ++u) {
+        if (u + 1 < units) ok = issue_s(u + 1);
+        if (ok) ok = issue_pv(u);
       }
       if (!ok && lane == 0) record_status(status, ELASTO_ERR_TIMEOUT);
       if (issued) {  // every MMA this thread issued has finished once `drain` completes
@@ -199,108 +286,74 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else {
     // ------------------------------------------------------------ softmax + epilogue
-    const int t = (warp - 2) >> 2;           // query tile of this group
-    const int qq = warp & 3;                 // TMEM lane quarter
-    const int r = qq * 32 + lane;            // row within the query tile
-    // a warp whose 32 rows are all past n has no softmax or read-out work
-    const bool active = t * QT + qq * 32 < n;
-    if (t < tiles) {
-      const uint32_t lane_base = tmem + (static_cast<uint32_t>(qq * 32) << 16) + t * 256;
-      const float kscale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
-      const int n_read = (n + 63) & ~63;                  // columns read in 64-column steps
-      for (int k = 0; k < nk; ++k) {
-        const int item = blockIdx.x + k * gridDim.x;
-        const uint32_t ph = k & 1;
-        const int b = (items - 1 - item) / heads, jj = (items - 1 - item) - b * heads;
-        if (!mbar_wait(&s_full[t], ph)) {
+    const int g = (warp - 2) >> 2;           // group: units g, g + 2, ...
+    const int qq = warp & 3;                 // TMEM lane quarter: rows 32 qq .. 32 qq + 31 of the tile
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(qq * 32) << 16) + g * 256;
+    uint8_t* const stage = obuf + (warp - 2) * O_BYTES;
+    {
+      for (int u = g; u < units; u += 2) {
+        const int k = tiles == 2 ? u >> 1 : u, t = tiles == 2 ? u & 1 : 0;
+        const uint32_t ph = (u >> 1) & 1;
+        // a warp whose 32 rows are all past n has no softmax or read-out work
+        const bool active = t * QT + qq * 32 < n;
+        if (!__all_sync(0xffffffffu, mbar_wait(&s_full[g], ph))) {
           if (lane == 0) record_status(status, ELASTO_ERR_TIMEOUT);
           break;
         }
         tc_fence_after();
         float sum = 1.0f;
         if (active) {
-          // pass 1: row max over the valid keys (four independent partial maxima)
-          float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-          for (int c = 0; c < n_read; c += 64) {
-            uint32_t v[32], u[32];
-            tmem_ld_32x32b_x32(lane_base + c, v);
-            tmem_ld_32x32b_x32(lane_base + c + 32, u);
-            tmem_ld_wait();
-            if (c + 64 <= n) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(v[j]));
-                m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(u[j]));
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) {
-                if (c + j < n) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(v[j]));
-                if (c + 32 + j < n) m4[j & 3] = fmaxf(m4[j & 3], __uint_as_float(u[j]));
-              }
-            }
+          switch (n >> 6) {  // whole 64-key chunks
+            case 0: sum = softmax_row<0>(lane_base, n); break;
+            case 1: sum = softmax_row<1>(lane_base, n); break;
+            case 2: sum = softmax_row<2>(lane_base, n); break;
+            case 3: sum = softmax_row<3>(lane_base, n); break;
+            default: sum = softmax_row<4>(lane_base, n); break;
           }
-          const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-          // pass 2: numerators and row sum; P as bf16 pairs into TMEM columns
-          // [c/2, c/2 + 32), all of which this pass has already read
-          const float mxs = mx * kscale;
-          float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-          for (int c = 0; c < n_read; c += 64) {
-            uint32_t v[64], pk[32];
-            tmem_ld_32x32b_x32(lane_base + c, *reinterpret_cast<uint32_t(*)[32]>(v));
-            tmem_ld_32x32b_x32(lane_base + c + 32, *reinterpret_cast<uint32_t(*)[32]>(v + 32));
-            tmem_ld_wait();
-            if (c + 64 <= n) {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                const float p0 = ex2_approx(fmaf(__uint_as_float(v[j]), kscale, -mxs));
-                const float p1 = ex2_approx(fmaf(__uint_as_float(v[j + 1]), kscale, -mxs));
-                s4[(j >> 1) & 3] += p0 + p1;
-                pk[j >> 1] = pack_bf16x2(p0, p1);
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 64; j += 2) {
-                const float p0 = (c + j < n) ? ex2_approx(fmaf(__uint_as_float(v[j]), kscale, -mxs)) : 0.0f;
-                const float p1 = (c + j + 1 < n) ? ex2_approx(fmaf(__uint_as_float(v[j + 1]), kscale, -mxs)) : 0.0f;
-                s4[(j >> 1) & 3] += p0 + p1;
-                pk[j >> 1] = pack_bf16x2(p0, p1);
-              }
-            }
-            tmem_st_16(lane_base + (c >> 1), *reinterpret_cast<const uint32_t(*)[16]>(pk));
-            tmem_st_16(lane_base + (c >> 1) + 16, *reinterpret_cast<const uint32_t(*)[16]>(pk + 16));
-          }
-          sum = (s4[0] + s4[1]) + (s4[2] + s4[3]);
           tmem_st_wait();
         }
         tc_fence_before();
-        mbar_arrive(&p_full[t]);
+        mbar_arrive(&p_full[g]);
         // epilogue
-        if (!mbar_wait(&o_full[t], ph)) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&o_full[g], ph))) {
           if (lane == 0) record_status(status, ELASTO_ERR_TIMEOUT);
           break;
         }
         tc_fence_after();
-        uint32_t o[64];
+        uint32_t o[2][32];
         if (active) {
-          tmem_ld_32x32b_x32(lane_base + O_COL, *reinterpret_cast<uint32_t(*)[32]>(o));
-          tmem_ld_32x32b_x32(lane_base + O_COL + 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32));
+          load64(lane_base + O_COL, o);
           tmem_ld_wait();
         }
         tc_fence_before();
-        mbar_arrive(&o_empty[t]);
-        const int row = t * QT + r;
-        if (active && row < n) {
+        mbar_arrive(&o_empty[g]);
+        if (active) {
           const float inv = 1.0f / sum;
-          uint4* dst = reinterpret_cast<uint4*>(out + (static_cast<size_t>(b) * n + row) * w + jj * HD);
+          const float2 inv2 = make_float2(inv, inv);
+          if (elect_one()) bulk_wait_read<0>();  // the staging's previous store has read it
+          __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            dst[j] = make_uint4(pack_bf16x2(__uint_as_float(o[8 * j + 0]) * inv, __uint_as_float(o[8 * j + 1]) * inv),
-                                pack_bf16x2(__uint_as_float(o[8 * j + 2]) * inv, __uint_as_float(o[8 * j + 3]) * inv),
-                                pack_bf16x2(__uint_as_float(o[8 * j + 4]) * inv, __uint_as_float(o[8 * j + 5]) * inv),
-                                pack_bf16x2(__uint_as_float(o[8 * j + 6]) * inv, __uint_as_float(o[8 * j + 7]) * inv));
+          for (int j = 0; j < 8; ++j) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int c = 8 * (j & 3) + 2 * i;
+              const float2 x = mul2(make_float2(__uint_as_float(o[j >> 2][c]), __uint_as_float(o[j >> 2][c + 1])), inv2);
+              pk[i] = pack_bf16x2(x.x, x.y);
+            }
+            *reinterpret_cast<uint4*>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (elect_one()) {
+            const int item = items - 1 - (blockIdx.x + k * gridDim.x), b = item / heads;
+            tma_store_3d(&tmO, stage, (item - b * heads) * HD, t * QT + qq * 32, b);
+            bulk_commit();
+          }
         }
       }
+      if (elect_one()) bulk_wait_all();
     }
   }
   __syncthreads();
@@ -338,7 +391,9 @@ elasto_status attn_plan(AttnPlan* p, const bf16* qkv, bf16* out, int batch_cap, 
   p->batch_cap = batch_cap;
   p->status = status;
   const uint64_t cols = static_cast<uint64_t>(3) * heads * HD;
+  const uint64_t ocols = static_cast<uint64_t>(heads) * HD;
   if (!encode_tmap_3d(&p->tmQ, qkv, cols, n, batch_cap, cols * 2, cols * 2 * n, HD, QT, 1) ||
+      !encode_tmap_3d(&p->tmO, out, ocols, n, batch_cap, ocols * 2, ocols * 2 * n, HD, 32, 1) ||
       !encode_tmap_3d(&p->tmKV, qkv, cols, n, batch_cap, cols * 2, cols * 2 * n, HD, p->n_pad, 1)) {
     set_error("attention: cuTensorMapEncodeTiled failed");
     return ELASTO_ERR_UNSUPPORTED;
@@ -351,7 +406,7 @@ cudaError_t attn_launch(const AttnPlan& p, int batch, cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
   const int items = batch * p.heads;
   const int grid = items < num_sms() ? items : num_sms();
-  return launch_pdl(attn_tc_kernel, dim3(grid), dim3(THREADS), smem_bytes_for(p.n_pad), s, p.tmQ, p.tmKV, p.out, p.n,
+  return launch_pdl(attn_tc_kernel, dim3(grid), dim3(THREADS), smem_bytes_for(p.n_pad), s, p.tmQ, p.tmKV, p.tmO, p.n,
                     p.n_pad,
                     p.heads, items, p.blk_stride, p.head_stride, p.status);
 }

@@ -255,7 +255,7 @@ cudaError_t halo_init_attributes();
 
 // ---------------------------------------------------------------- attention
 struct AttnPlan {
-  CUtensorMap tmQ, tmKV;
+  CUtensorMap tmQ, tmKV, tmO;  // tmO: out, boxes of 64 columns x 32 rows of one image
   const bf16* qkv;
   bf16* out;
   int n, n_pad, heads, batch_cap;

@@ -129,13 +129,6 @@ __device__ __forceinline__ void copy_phase(PkPhase* dst, const PkPhase* src, int
 constexpr int PK_Q_OFF = 0, PK_K_OFF = 16384, PK_V_OFF = 16384 + 256 * 128;
 static_assert(PK_V_OFF + 256 * 128 <= PK_RING, "attention buffers fit the ring");
 
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, const void* src, int x, int y, int z) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];" ::"l"(
-                   reinterpret_cast<uint64_t>(tm)),
-               "r"(smem_addr(src)), "r"(x), "r"(y), "r"(z)
-               : "memory");
-}
-
 // One thread's row piece (nch <= 8 chunks of 16 bytes) into its warp's
 // staging box of 32 such rows, the layout the TMA store reads: dense rows,
 // and for 128-byte rows the 128-byte swizzle (chunk c of row r at c ^ (r % 8),
