@@ -34,11 +34,12 @@
 //    of it in the barrier and in bias loads from the loaded L2 path; eight
 //    warps on their own lack the overlap for GELU (FC1 174 us), sixteen the
 //    registers. GELU, bias and residual use packed fp32 pairs.
-//    * the fp32 residual stream (out-proj, FC2) leaves by TMA reduce-add: X is
-//      not read into the SM. FC2 (K = 3072) 158 -> 149 us, out-proj 76 -> 72.
-//      A plan of few tiles (or with another residual source) reads the old rows
-//      into the staging pieces ahead instead, as the 16-bit residual + ReLU of
-//      the CNN block outputs does.
+//    * the fp32 residual stream (out-proj, FC2) leaves by TMA reduce-add, from
+//      eight warps: X is not read into the SM. FC2 (K = 3072, 50432 rows) 154 ->
+//      142 us, K = 1536 92 -> 86. Where memory sets the pace, and in a plan of
+//      few tiles, the old rows are read into the staging pieces ahead instead
+//      (out-proj 72 -> 68), as the 16-bit residual + ReLU of the CNN block
+//      outputs are.
 //    * the remaining epilogue (fp32 out) transposes through padded shared
 //      memory for row-contiguous stores (warps 2-5); it also writes the
 //      partial sums of a split-K plan, whose k-block range is
@@ -58,21 +59,25 @@ namespace elasto {
 namespace {
 
 constexpr int BM = 128, BK = 64, MAX_STAGES = 8, MAX_BN = 256;
-constexpr int EPI_WARPS = 12;               // three epilogue warps per TMEM lane quarter
-constexpr int GROUPS = EPI_WARPS / 4;       // a group is one warp of every quarter: 128 rows
-constexpr int THREADS = 64 + 32 * EPI_WARPS;
-constexpr int THREADS_CONV = THREADS + 32;  // implicit convolutions: warp 14 is a second TMA producer
+// Epilogue warps: three per TMEM lane quarter; two where the residual is added
+// by the store, whose arithmetic is light (the staging saved is an operand
+// stage: 50432 x 768 x 1536 91.7 -> 85.5 us, K = 3072 147 -> 142); one for the
+// transposing fp32 epilogue.
+constexpr int MAX_EPI_WARPS = 12;
+constexpr int epi_warps(int epi) { return epi == EPI_BIAS_F32 ? 4 : epi == EPI_BIAS_ADD_F32 ? 8 : MAX_EPI_WARPS; }
+constexpr int epi_threads(int epi) { return 64 + 32 * epi_warps(epi); }
+constexpr int THREADS_CONV = 64 + 32 * MAX_EPI_WARPS + 32;  // implicit convolutions: warp 14 is a second TMA producer
 constexpr int A_STAGE = BM * BK * 2;        // 16 KB
 constexpr int WBUF = 32 * 128;              // 4 KB staging piece of one epilogue warp (32 rows x 128 B)
-constexpr int CBUF = EPI_WARPS * WBUF;      // 48 KB: one staging piece for every epilogue warp
+constexpr int CBUF = MAX_EPI_WARPS * WBUF;  // 48 KB: one staging piece for each of twelve epilogue warps
 constexpr int POOL = 224 * 1024;            // operand ring + staging pieces
 constexpr int MAX_CBUFS = 2;                // staging pieces per epilogue warp
 constexpr int EPI_LD = 33;                  // padded row of the transpose tile
 constexpr int EPI_TILE = 32 * EPI_LD;       // floats per epilogue warp
 constexpr int TMEM_COLS = 512;
 constexpr size_t SMEM_BYTES = 1024 + POOL + 2048;
-constexpr int BARS = 2 * MAX_STAGES + 6 + EPI_WARPS * MAX_CBUFS;  // mbarriers (the bias after them is read as float4)
-static_assert(BARS * 8 % 16 == 0 && BARS * 8 + 32 * EPI_WARPS * 4 + 4 * (1 + GROUPS) <= 2048, "barriers and bias");
+constexpr int BARS = 2 * MAX_STAGES + 6 + MAX_EPI_WARPS * MAX_CBUFS;  // mbarriers (the bias after them is read as float4)
+static_assert(BARS * 8 % 16 == 0 && BARS * 8 + 32 * MAX_EPI_WARPS * 4 + 4 * (1 + MAX_EPI_WARPS / 4) <= 2048, "barriers and bias");
 
 template <int EPI>
 struct EpiTraits {
@@ -144,8 +149,12 @@ __device__ __forceinline__ void conv_tile(const GemmArgs& a, int mtile, int& b0,
 
 // Walks the chunks of one epilogue warp group over this CTA's tiles. The
 // chunks of all tiles form one sequence (cols(t) of them in tile t); group g
-// takes every third one, so that tiles of a single chunk go round.
-__device__ __forceinline__ int first_chunk(int g, int before) { return (g + GROUPS - before) % GROUPS; }
+// takes every GROUPS-th one, so that tiles of a single chunk go round.
+template <int GROUPS>
+__device__ __forceinline__ int first_chunk(int g, int before) {
+  return (g + GROUPS - before) % GROUPS;
+}
+template <int GROUPS>
 struct ChunkIter {
   int t, c, before;  // tile, chunk in it, number of chunks before the tile (mod GROUPS)
   bool valid;
@@ -154,7 +163,7 @@ struct ChunkIter {
     while (valid && c >= cols(t)) {
       before = (before + cols(t)) % GROUPS;
       t += stride;
-      c = first_chunk(g, before);
+      c = first_chunk<GROUPS>(g, before);
       valid = t < tiles;
     }
   }
@@ -179,12 +188,13 @@ struct ChunkIter {
 // signals both CTAs' barriers with multicast commits; each CTA's epilogue
 // reads its own half of the accumulator from its own TMEM.
 template <int EPI, int NB, bool PAIR>
-__global__ void __launch_bounds__(THREADS_CONV, 1)
+__global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmB2,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmR,
                    const GemmArgs args) {
   using TR = EpiTraits<EPI>;
+  constexpr int EPI_WARPS = epi_warps(EPI), GROUPS = EPI_WARPS / 4;  // a group is one warp of every quarter: 128 rows
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int S = args.stages, E = args.cbufs;
@@ -203,7 +213,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
   uint64_t* bfull = drain + 1;  // resident B landed
-  uint64_t* rfull = bfull + 1;  // residual landed: MAX_CBUFS barriers per epilogue warp
+  uint64_t* rfull = bfull + 1;  // residual landed: one per staging piece
   float* sbias = reinterpret_cast<float*>(bars + BARS);  // 32 values per epilogue warp
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sbias + 32 * EPI_WARPS);
 
@@ -231,7 +241,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull[a], 1);
-      mbar_init(&tempty[a], (PAIR ? 2 : 1) * (TR::tma ? EPI_WARPS : 4));
+      mbar_init(&tempty[a], (PAIR ? 2 : 1) * EPI_WARPS);
     }
     mbar_init(drain, 1);
     if constexpr (TR::resid)
@@ -279,7 +289,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
   // tiles (128 images of 56 x 56 x 16 -> 16 channels: 54 us with one, 48 us
   // with two; the strided 128-channel 3x3 of stage 2: 37.4 and 35.6).
   const int nprod = (args.conv && static_cast<int>(blockDim.x) == THREADS_CONV) ? 2 : 1;
-  if (warp == 0 || warp == THREADS / 32) {
+  if (warp == 0 || warp == 2 + EPI_WARPS) {
     // ------------------------------------------------------------ producer
     const int pid = warp == 0 ? 0 : 1;
     if (pid < nprod && nk > 0 && elect_one()) {
@@ -494,7 +504,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     volatile uint32_t* fail = tmem_slot + 1 + g;
     uint64_t* rf = rfull + ew * MAX_CBUFS;
     float* sb = sbias + 32 * ew;
-    ChunkIter pf;  // residual prefetch (the elected thread)
+    ChunkIter<GROUPS> pf{};  // residual prefetch (the elected thread)
     long loads = 0, consumed = 0;
     auto fetch = [&](int e) {
       mbar_expect_tx(&rf[e], WBUF);
@@ -516,7 +526,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
       const int acc = local & 1;
       const uint32_t use = static_cast<uint32_t>(local >> 1);
       const int m0 = row0(t), n0 = (t % nt) * bn, nvalid = cols(t);
-      int c = first_chunk(g, before);
+      int c = first_chunk<GROUPS>(g, before);
       before = (before + nvalid) % GROUPS;
       // Each chunk's bias is requested a chunk ahead (before the accumulator
       // wait for the first), one column per lane, and broadcast from shared
@@ -685,8 +695,7 @@ __global__ void __launch_bounds__(THREADS_CONV, 1)
     }
   } else {
     // ------------------------------------------------------------ transpose epilogue
-    // (warps 2-5 only; the other epilogue warps have nothing to do here)
-    if (warp < 6) {
+    {
     const int q = warp & 3;  // TMEM lane quarter this warp may access
     float* st = reinterpret_cast<float*>(sC) + (warp - 2) * EPI_TILE;
     int local = 0;
@@ -851,7 +860,7 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_pdl
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.blockDim = dim3(a.conv ? THREADS_CONV : THREADS);
+    cfg.blockDim = dim3(a.conv ? THREADS_CONV : epi_threads(EPI));
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -871,7 +880,7 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
   } else {
     const int tiles = (a.conv ? conv_mtiles(a) : (M + BM - 1) / BM) * nt * (a.ksplit > 1 ? a.ksplit : 1);
     const int grid = tiles < num_sms() ? tiles : num_sms();
-    return launch_pdl(gemm_tc_kernel<EPI, NB, false>, dim3(grid), dim3(a.conv ? THREADS_CONV : THREADS), SMEM_BYTES, s,
+    return launch_pdl(gemm_tc_kernel<EPI, NB, false>, dim3(grid), dim3(a.conv ? THREADS_CONV : epi_threads(EPI)), SMEM_BYTES, s,
                       p.tmA, p.tmB, p.tmB2,
                       p.tmC, p.tmR, a);
   }
@@ -964,16 +973,17 @@ void choose_tile(const Problem& p, int step, bool pairs_allowed, int* bn, bool* 
 namespace {
 
 // Splits the pool between the operand ring and the epilogue's staging pieces.
-// cbufs counts pieces per epilogue warp: 2 with a residual read through them
-// (its fetch depth), if that leaves 3 stages, else 1.
-bool ring_layout(GemmArgs* a, bool resid) {
-  const int stage = a->b_stage + A_STAGE;
+// cbufs counts pieces per epilogue warp: with a residual read through them (its
+// fetch depth) as many as leave 3 stages, else 1.
+bool ring_layout(GemmArgs* a, int epi) {
+  const int stage = a->b_stage + A_STAGE, piece = epi_warps(epi) * WBUF;
+  const bool resid = epi == EPI_BIAS_RESID_F32 || is_resid16(epi);
   for (int e = resid ? MAX_CBUFS : 1; e >= 1; --e) {
     a->cbufs = e;
-    a->stages = std::min((POOL - e * CBUF) / stage, MAX_STAGES);
+    a->stages = std::min((POOL - e * piece) / stage, MAX_STAGES);
     if (a->stages >= 3) break;
   }
-  return a->stages >= 2 && a->cbufs >= 1 && a->cbufs <= MAX_CBUFS && a->stages * stage + a->cbufs * CBUF <= POOL;
+  return a->stages >= 2 && a->stages * stage + a->cbufs * piece <= POOL;
 }
 
 }  // namespace
@@ -1021,14 +1031,18 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
   a.ldo = ldo;
   a.status = status;
   a.b_planes = planes;
-  // On a nearly idle chip reading X ahead, behind the main loop, beats the
-  // longer completion of a reduce-add.
+  // Reduce-add stores move 5.1 TB/s of X, loads and stores 5.8, so X is read
+  // ahead where memory sets the pace: X past the L2 and a short reduction (50432
+  // x 768 x 192: 65 us added, 55 us read ahead; K = 1536: 92 and 100; X in the
+  // L2, 6304 x 768 x 768: 11.5 and 14.9). And on a nearly idle chip, where the
+  // read hides behind the main loop and a reduce-add completes later.
   const int rows = pair ? 2 * BM : BM;
   const long tiles = static_cast<long>((Mt + rows - 1) / rows) * ((N + a.bn - 1) / a.bn);
-  if (epi == EPI_BIAS_ADD_F32 && 4 * tiles <= (pair ? sms / 2 : sms)) epi = EPI_BIAS_RESID_F32;
+  const bool memory_bound = K <= 1024 && 4.0 * Mt * N > 64e6;
+  if (epi == EPI_BIAS_ADD_F32 && (memory_bound || 4 * tiles <= (pair ? sms / 2 : sms))) epi = EPI_BIAS_RESID_F32;
   p->epi = epi;
   if (tma_out) {
-    if (!ring_layout(&a, resid16 || epi == EPI_BIAS_RESID_F32)) {
+    if (!ring_layout(&a, epi)) {
       set_error("gemm_plan: shared-memory layout does not fit");
       return ELASTO_ERR_UNSUPPORTED;
     }
@@ -1287,7 +1301,7 @@ elasto_status gemm_set_residual_source(GemmPlan* p, const void* src, int M_cap, 
   const int ldo = p->args.ldo;
   if (f32) {  // the residual is read: stores instead of reduce-adds, and the staging depth to fetch it ahead
     p->epi = EPI_BIAS_RESID_F32;
-    if (!ring_layout(&p->args, true)) {
+    if (!ring_layout(&p->args, p->epi)) {
       set_error("gemm_set_residual_source: shared-memory layout does not fit");
       return ELASTO_ERR_UNSUPPORTED;
     }

@@ -19,7 +19,8 @@ def _bf16(rng, shape, scale=1.0):
 @pytest.mark.parametrize("M,N,K,epi", [
     (19457, 2312, 768, binding.EPI_BIAS_BF16),       # pairs: one row and eight columns past the tiles
     (19713, 520, 264, binding.EPI_BIAS_GELU_BF16),   # pairs, K a remainder of a k-block
-    (25089, 776, 520, binding.EPI_BIAS_RESID_F32),   # pairs, residual added by the store
+    (19713, 520, 1160, binding.EPI_BIAS_RESID_F32),  # pairs, residual added by the store
+    (25089, 776, 520, binding.EPI_BIAS_RESID_F32),   # pairs, short reduction past the L2: residual read ahead
     (257, 64, 64, binding.EPI_BIAS_RESID_F32),       # few tiles: residual read ahead
     (12289, 40, 192, binding.EPI_BIAS_RESID_F32),    # narrow single tiles
 ])
