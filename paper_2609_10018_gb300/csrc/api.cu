@@ -56,6 +56,7 @@ cudaError_t ensure_kernel_attributes() {
     if (r == cudaSuccess) r = halo_init_attributes();
     if (r == cudaSuccess) r = attn_init_attributes();
     if (r == cudaSuccess) r = cnn_init_attributes();
+    if (r == cudaSuccess) r = head_init_attributes();
     if (r == cudaSuccess) r = pk_init_attributes();
     g_attr_err[dev] = r;
   });

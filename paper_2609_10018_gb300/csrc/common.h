@@ -268,9 +268,7 @@ elasto_status attn_plan(AttnPlan* p, const bf16* qkv, bf16* out, int batch_cap, 
                         bool interleaved = false);
 cudaError_t attn_launch(const AttnPlan& p, int batch, cudaStream_t s);
 cudaError_t attn_init_attributes();
-// The CNN classifier's shared-memory limit (its pooled rows: 8 x d fp32, up
-// to d = kCnnMaxFeatures).
-constexpr int kCnnMaxFeatures = 4096;
+constexpr int kCnnFeatures = 2048;  // pooled features of ResNet-50
 cudaError_t cnn_init_attributes();
 
 // ---------------------------------------------------------------- small kernels
@@ -291,6 +289,7 @@ cudaError_t token_addend_launch(const float* cls, const float* pos, const float*
                                 float* dst, cudaStream_t s);
 // logits[b, c] = LN(X[b * n, :]) . head_w[c, :] + head_b[c], all fp32; rows of
 // width d, LayerNorm statistics over the first d_true channels (the rest zero).
+cudaError_t head_init_attributes();
 cudaError_t head_launch(const float* X, int B, int n, int d, int d_true, const float* g, const float* b, const float* Wh,
                         const float* bh, int C, float* logits, cudaStream_t s);
 // gathers for create-time packing

@@ -15,6 +15,7 @@
 
 #include <cudaTypedefs.h>
 
+#include "classifier.cuh"
 #include "common.h"
 #include "ptx.cuh"
 
@@ -236,26 +237,37 @@ namespace {
 
 // A [B * n, K] in token order, K = P*P*C in (ky, kx, c) order. One thread per
 // 16-byte piece (8 bf16): within a patch row, the P*C values (kx, c) are
-// contiguous in the NHWC image, so a piece is one aligned 16-byte copy.
-__global__ void patch_rows_vec_kernel(const bf16* __restrict__ img, int B, int H, int W, int C, int P,
-                                      uint4* __restrict__ A) {
+// contiguous in the NHWC image, so a piece is one aligned 16-byte copy. Four
+// pieces a thread are in flight at once, and their places are found in 32-bit
+// arithmetic (Idx) where it reaches: 64-bit divisions and single copies took 38
+// us for 256 images of 224 x 224 (154 MB), now 29.
+template <typename Idx>
+__global__ void __launch_bounds__(256) patch_rows_vec_kernel(const bf16* __restrict__ img, int B, int H, int W, int C,
+                                                             int P, uint4* __restrict__ A) {
   pdl_wait();
   pdl_trigger();
-  const int gw = W / P, np = (H / P) * gw, n = np + 1, K = P * P * C;
-  const int row_pieces = K / 8, seg = P * C / 8;  // pieces per A row, per patch row
-  const size_t total = static_cast<size_t>(B) * n * row_pieces;
-  for (size_t t = static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < total;
-       t += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    const int j = static_cast<int>(t % row_pieces);
-    const size_t row = t / row_pieces;
-    const int tok = static_cast<int>(row % n), bb = static_cast<int>(row / n);
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (tok > 0) {
-      const int p = tok - 1, ky = j / seg, jj = j - ky * seg;
-      const int yy = (p / gw) * P + ky, x0 = (p % gw) * P;
-      v = *reinterpret_cast<const uint4*>(img + ((static_cast<size_t>(bb) * H + yy) * W + x0) * C + jj * 8);
+  const int gw = W / P, np = (H / P) * gw;
+  const Idx n = np + 1, row_pieces = P * P * C / 8;
+  const int seg = P * C / 8;  // pieces per patch row
+  const Idx total = static_cast<Idx>(B) * n * row_pieces, step = static_cast<Idx>(gridDim.x) * blockDim.x;
+  for (Idx t = static_cast<Idx>(blockIdx.x) * blockDim.x + threadIdx.x; t < total; t += 4 * step) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const Idx tt = t + u * step;
+      v[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (tt >= total) continue;
+      const Idx row = tt / row_pieces, bb = row / n;
+      const int j = static_cast<int>(tt - row * row_pieces), tok = static_cast<int>(row - bb * n);
+      if (tok > 0) {
+        const int p = tok - 1, ky = j / seg, jj = j - ky * seg;
+        const int py = p / gw, yy = py * P + ky, x0 = (p - py * gw) * P;
+        v[u] = __ldg(reinterpret_cast<const uint4*>(img + ((static_cast<size_t>(bb) * H + yy) * W + x0) * C + jj * 8));
+      }
     }
-    A[t] = v;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * step < total) A[t + u * step] = v[u];
   }
 }
 
@@ -306,8 +318,13 @@ cudaError_t patch_rows_launch(const void* images, int img_dtype, int B, int H, i
   const int n = (H / P) * (W / P) + 1, K = P * P * C;
   if (img_dtype == ELASTO_BF16 && (P * C) % 8 == 0) {
     const size_t total = static_cast<size_t>(B) * n * (K / 8);
-    return launch_pdl(patch_rows_vec_kernel, dim3(grid_1d(total)), dim3(256), 0, s, static_cast<const bf16*>(images),
-                      B, H, W, C, P, reinterpret_cast<uint4*>(A));
+    // few pieces: one a thread, on more SMs (the loop's other three are past the end)
+    const dim3 grid(grid_1d(total < 300000 ? total : (total + 3) / 4));
+    const bf16* img = static_cast<const bf16*>(images);
+    uint4* dst = reinterpret_cast<uint4*>(A);
+    if (total < (1u << 29))  // t + 4 * step stays below 2^32
+      return launch_pdl(patch_rows_vec_kernel<uint32_t>, grid, dim3(256), 0, s, img, B, H, W, C, P, dst);
+    return launch_pdl(patch_rows_vec_kernel<size_t>, grid, dim3(256), 0, s, img, B, H, W, C, P, dst);
   }
   const unsigned blocks = grid_1d(static_cast<size_t>(B) * n * K);
   if (img_dtype == ELASTO_BF16)
@@ -325,85 +342,14 @@ cudaError_t token_addend_launch(const float* cls, const float* pos, const float*
 }
 
 // ---------------------------------------------------------------- classifier
-namespace {
-
-constexpr int HEAD_IMGS = 8;                  // class-token rows per CTA
-constexpr int HEAD_CPW = 4;                   // classes per warp, computed together
-constexpr int HEAD_CLASSES = 8 * HEAD_CPW;    // classes per CTA
-
-// grid (ceil(B / 8), ceil(C / 32)), 256 threads: LayerNorm of up to 8 class
-// tokens into shared memory (fp32), then each warp computes 4 classes x 8
-// images of dot products at once: every normalised float4 it reads from shared
-// memory feeds 16 FMAs, every classifier float4 32.
-// d is the row width of X and Wh; the LayerNorm statistics cover the first
-// d_true channels (the rest are the zero padding of a pruned width).
-__global__ void __launch_bounds__(256) head_kernel(const float* __restrict__ X, int B, int n, int d, int d_true,
-                                                   const float* __restrict__ g, const float* __restrict__ bta,
-                                                   const float* __restrict__ Wh, const float* __restrict__ bh, int C,
-                                                   float* __restrict__ logits) {
-  pdl_wait();
-  pdl_trigger();
-  extern __shared__ float sy[];  // [HEAD_IMGS][d]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b0 = blockIdx.x * HEAD_IMGS;
-  const int nimg = min(HEAD_IMGS, B - b0);
-  if (warp < nimg) {
-    const float* xr = X + static_cast<size_t>(b0 + warp) * n * d;  // class token row
-    float s = 0.0f;
-    for (int c = lane; c < d_true; c += 32) s += xr[c];
-    const float mean = warp_sum(s) / d_true;
-    float ss = 0.0f;
-    for (int c = lane; c < d_true; c += 32) {
-      const float a = xr[c] - mean;
-      ss += a * a;
-    }
-    const float rstd = rsqrtf(warp_sum(ss) / d_true + 1e-6f);
-    for (int c = lane; c < d; c += 32) sy[warp * d + c] = c < d_true ? (xr[c] - mean) * rstd * g[c] + bta[c] : 0.0f;
-  }
-  __syncthreads();
-  const int c0 = blockIdx.y * HEAD_CLASSES + warp * HEAD_CPW;
-  if (c0 >= C) return;
-  const float* wr[HEAD_CPW];
-#pragma unroll
-  for (int j = 0; j < HEAD_CPW; ++j) wr[j] = Wh + static_cast<size_t>(min(c0 + j, C - 1)) * d;
-  float acc[HEAD_CPW][HEAD_IMGS];
-#pragma unroll
-  for (int j = 0; j < HEAD_CPW; ++j)
-#pragma unroll
-    for (int i = 0; i < HEAD_IMGS; ++i) acc[j][i] = 0.0f;
-#pragma unroll 2
-  for (int c = lane * 4; c < d; c += 128) {
-    float4 wv[HEAD_CPW];
-#pragma unroll
-    for (int j = 0; j < HEAD_CPW; ++j) wv[j] = *reinterpret_cast<const float4*>(wr[j] + c);
-#pragma unroll
-    for (int i = 0; i < HEAD_IMGS; ++i) {
-      if (i < nimg) {
-        const float4 yv = *reinterpret_cast<const float4*>(sy + i * d + c);
-#pragma unroll
-        for (int j = 0; j < HEAD_CPW; ++j)
-          acc[j][i] += wv[j].x * yv.x + wv[j].y * yv.y + wv[j].z * yv.z + wv[j].w * yv.w;
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < HEAD_CPW; ++j)
-#pragma unroll
-    for (int i = 0; i < HEAD_IMGS; ++i) {
-      const float v = warp_sum(acc[j][i]);
-      if (lane == 0 && i < nimg && c0 + j < C) logits[static_cast<size_t>(b0 + i) * C + c0 + j] = v + bh[c0 + j];
-    }
-}
-
-}  // namespace
+cudaError_t head_init_attributes() { return classifier::init_attributes<true, 8>(1024); }
 
 cudaError_t head_launch(const float* X, int B, int n, int d, int d_true, const float* g, const float* b,
                         const float* Wh, const float* bh, int C, float* logits, cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
-  if (d % 4 != 0 || d_true <= 0 || d_true > d) return cudaErrorInvalidValue;
-  dim3 grid((B + HEAD_IMGS - 1) / HEAD_IMGS, (C + HEAD_CLASSES - 1) / HEAD_CLASSES);
-  return launch_pdl(head_kernel, grid, dim3(256), HEAD_IMGS * d * sizeof(float), s, X, B, n, d, d_true, g, b, Wh, bh,
-                    C, logits);
+  if (d % 4 != 0 || d > 1024 || d_true <= 0 || d_true > d) return cudaErrorInvalidValue;
+  // the class token is each image's first row
+  return classifier::launch<true, 8>(X, static_cast<size_t>(n) * d, B, d, d_true, g, b, Wh, bh, C, logits, s);
 }
 
 // ---------------------------------------------------------------- packing
