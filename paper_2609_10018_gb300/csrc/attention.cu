@@ -159,8 +159,8 @@ __device__ __forceinline__ float softmax_row(uint32_t tm, int n) {
 
 __global__ void __launch_bounds__(THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV,
-                   const __grid_constant__ CUtensorMap tmO, int n, int n_pad, int heads, int items, int blk_stride,
-                   int head_stride, int* status) {
+                   const __grid_constant__ CUtensorMap tmO, int n, int n_pad, int heads, int items, int split,
+                   int blk_stride, int head_stride, int* status) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int ns = kv_slots_for(n_pad);
@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
 
   const int warp = warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const int tiles = n > QT ? 2 : 1;
+  // split: an item is one query tile of an (image, head), item & 1
+  const int tiles = n > QT && !split ? 2 : 1;
   // items of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
   const int nk = items > static_cast<int>(blockIdx.x) ? (items - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   // unit u: query tile u % tiles of item u / tiles, worked on by group u & 1
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       int k = 0;
       for (; k < nk; ++k) {
         const int item = blockIdx.x + k * gridDim.x;
-        const int slot = k % ns, b = (items - 1 - item) / heads, jj = (items - 1 - item) - b * heads;
+        const int slot = k % ns, r = items - 1 - item, bh = split ? r >> 1 : r, b = bh / heads, jj = bh - b * heads;
         if (!mbar_wait(&kv_empty[slot], ((k / ns) & 1) ^ 1) || !mbar_wait(&q_empty[k & 1], ((k >> 1) & 1) ^ 1)) {
           ok = false;
           break;
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         tma_load_3d(kb, &tmKV, &full[slot], qx + blk_stride, 0, b);
         tma_load_3d(kb + slot_bytes / 2, &tmKV, &full[slot], qx + 2 * blk_stride, 0, b);
         for (int t = 0; t < tiles; ++t)
-          tma_load_3d(qbuf + (2 * t + (k & 1)) * Q_BYTES, &tmQ, &full[slot], qx, t * QT, b);
+          tma_load_3d(qbuf + (2 * t + (k & 1)) * Q_BYTES, &tmQ, &full[slot], qx, (split ? r & 1 : t) * QT, b);
       }
       if (!ok) record_status(status, ELASTO_ERR_TIMEOUT);
       // the loads of the last items have landed before the CTA exits
@@ -292,7 +293,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint8_t* const stage = obuf + (warp - 2) * O_BYTES;
     {
       for (int u = g; u < units; u += 2) {
-        const int k = tiles == 2 ? u >> 1 : u, t = tiles == 2 ? u & 1 : 0;
+        const int k = tiles == 2 ? u >> 1 : u;
+        const int item = items - 1 - (blockIdx.x + k * gridDim.x);
+        const int t = tiles == 2 ? u & 1 : split ? item & 1 : 0;
         const uint32_t ph = (u >> 1) & 1;
         // a warp whose 32 rows are all past n has no softmax or read-out work
         const bool active = t * QT + qq * 32 < n;
@@ -347,8 +350,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           fence_async_smem();
           __syncwarp();
           if (elect_one()) {
-            const int item = items - 1 - (blockIdx.x + k * gridDim.x), b = item / heads;
-            tma_store_3d(&tmO, stage, (item - b * heads) * HD, t * QT + qq * 32, b);
+            const int bh = split ? item >> 1 : item, b = bh / heads;
+            tma_store_3d(&tmO, stage, (bh - b * heads) * HD, t * QT + qq * 32, b);
             bulk_commit();
           }
         }
@@ -404,11 +407,13 @@ elasto_status attn_plan(AttnPlan* p, const bf16* qkv, bf16* out, int batch_cap, 
 
 cudaError_t attn_launch(const AttnPlan& p, int batch, cudaStream_t s) {
   if (batch <= 0) return cudaSuccess;
-  const int items = batch * p.heads;
+  // where the chip would be half empty, a CTA takes one query tile instead of
+  // both (K and V are then loaded twice)
+  const int split = p.n > QT && 2 * batch * p.heads <= num_sms() ? 1 : 0;
+  const int items = batch * p.heads * (1 + split);
   const int grid = items < num_sms() ? items : num_sms();
   return launch_pdl(attn_tc_kernel, dim3(grid), dim3(THREADS), smem_bytes_for(p.n_pad), s, p.tmQ, p.tmKV, p.tmO, p.n,
-                    p.n_pad,
-                    p.heads, items, p.blk_stride, p.head_stride, p.status);
+                    p.n_pad, p.heads, items, split, p.blk_stride, p.head_stride, p.status);
 }
 
 }  // namespace elasto

@@ -94,6 +94,9 @@ enum GemmEpi : int {
   // EPI_BIAS_RESID_F32 whose residual is the output itself: the tile leaves by
   // TMA reduce-add stores (gemm_plan picks it; gemm_set_residual_source undoes it)
   EPI_BIAS_ADD_F32 = 100,
+  // fp32 partial sums of a split reduction, [split][row][N] by TMA stores
+  // (gemm_plan_split_resid)
+  EPI_PART_F32 = 101,
 };
 
 struct GemmArgs {

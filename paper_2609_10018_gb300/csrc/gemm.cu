@@ -40,10 +40,11 @@
 //      few tiles, the old rows are read into the staging pieces ahead instead
 //      (out-proj 72 -> 68), as the 16-bit residual + ReLU of the CNN block
 //      outputs are.
-//    * the remaining epilogue (fp32 out) transposes through padded shared
-//      memory for row-contiguous stores (warps 2-5); it also writes the
-//      partial sums of a split-K plan, whose k-block range is
-//      tile / (mt * nt).
+//    * a split-K plan (k-block range tile / (mt * nt)) stores fp32 partial sums
+//      the same way; the transposing epilogue took its CTAs 2.5 us of a 4.9 us
+//      one-image launch.
+//    * the remaining epilogue (fp32 out, any row stride) transposes through
+//      padded shared memory for row-contiguous stores.
 //  - implicit-GEMM convolution: A tiles are 4-D TMA boxes of the NHWC input
 //    (one tap and channel group per k-block, padding read as zeros), and the
 //    output is stored by 4-D boxes of the tile's pixel block.
@@ -64,7 +65,9 @@ constexpr int BM = 128, BK = 64, MAX_STAGES = 8, MAX_BN = 256;
 // stage: 50432 x 768 x 1536 91.7 -> 85.5 us, K = 3072 147 -> 142); one for the
 // transposing fp32 epilogue.
 constexpr int MAX_EPI_WARPS = 12;
-constexpr int epi_warps(int epi) { return epi == EPI_BIAS_F32 ? 4 : epi == EPI_BIAS_ADD_F32 ? 8 : MAX_EPI_WARPS; }
+constexpr int epi_warps(int epi) {
+  return epi == EPI_BIAS_F32 ? 4 : epi == EPI_BIAS_ADD_F32 || epi == EPI_PART_F32 ? 8 : MAX_EPI_WARPS;
+}
 constexpr int epi_threads(int epi) { return 64 + 32 * epi_warps(epi); }
 constexpr int THREADS_CONV = 64 + 32 * MAX_EPI_WARPS + 32;  // implicit convolutions: warp 14 is a second TMA producer
 constexpr int A_STAGE = BM * BK * 2;        // 16 KB
@@ -86,9 +89,9 @@ struct EpiTraits {
   // brought into the staging buffer by TMA like the fp32 residual stream
   static constexpr bool resid16 = EPI == EPI_BIAS_RESID_RELU_BF16 || EPI == EPI_BIAS_RESID_RELU_F16;
   static constexpr bool tma = EPI == EPI_BIAS_BF16 || EPI == EPI_BIAS_GELU_BF16 || EPI == EPI_BIAS_RELU_BF16 ||
-                              EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32 || EPI == EPI_BIAS_RELU_F16 ||
-                              EPI == EPI_BIAS_F16 || resid16;
-  static constexpr bool f32 = EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32;
+                              EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32 || EPI == EPI_PART_F32 ||
+                              EPI == EPI_BIAS_RELU_F16 || EPI == EPI_BIAS_F16 || resid16;
+  static constexpr bool f32 = EPI == EPI_BIAS_RESID_F32 || EPI == EPI_BIAS_ADD_F32 || EPI == EPI_PART_F32;
   // the old value is read into the staging piece by TMA; EPI_BIAS_ADD_F32
   // reads nothing: the store itself adds to memory
   static constexpr bool resid = EPI == EPI_BIAS_RESID_F32 || resid16;
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
   // split-K (fp32 partial outputs only): tile t covers output tile
   // t % (mt * nt) and k-block range t / (mt * nt) of ks. Every other
   // epilogue has ks = 1 at compile time and no division on its tile path.
-  constexpr bool kSplit = EPI == EPI_BIAS_F32;
+  constexpr bool kSplit = EPI == EPI_PART_F32;
   const int ks = kSplit && args.ksplit > 1 ? args.ksplit : 1;
   const int mn_tiles = mt * nt;
   const int tiles = mn_tiles * ks;
@@ -490,10 +493,10 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
     const uint32_t row_tm = tmem_base + (static_cast<uint32_t>(q * 32) << 16);
     auto piece = [&](int e) { return sC + ((g * E + e) * 4 + q) * WBUF; };  // a group's four pieces are one 16 KB chunk
     auto cols = [&](int t) {
-      const int left = (N - (t % nt) * bn + CW - 1) / CW;
+      const int left = (N - (t % nt) * bn + CW - 1) / CW;  // (nt divides the tiles of a split)
       return left < cpt ? left : cpt;
     };
-    auto row0 = [&](int t) { return m_tile(args, t / nt, mt) * TM + rank * BM; };
+    auto row0 = [&](int t) { return m_tile(args, (kSplit ? t % mn_tiles : t) / nt, mt) * TM + rank * BM; };
     // Warps work on their own: each reads its 32 rows of its chunks, writes
     // them to its own staging pieces and stores them with its own 32-row TMA
     // boxes; the only hand-offs are the accumulator barriers. (Convolution
@@ -663,6 +666,8 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
             if (m0 + q * 32 < M) {
               if constexpr (EPI == EPI_BIAS_ADD_F32)
                 tma_add_2d(&tmC, piece(e), col, m0 + q * 32);
+              else if constexpr (kSplit)
+                tma_store_3d(&tmC, piece(e), col, m0 + q * 32, t / mn_tiles);
               else
                 tma_store_2d(&tmC, piece(e), col, m0 + q * 32);
             }
@@ -707,8 +712,7 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
         break;
       }
       tc_fence_after();
-      const int tq = t % mn_tiles;
-      const int m0 = m_tile(args, tq / nt, mt) * TM + rank * BM, n0 = (tq % nt) * bn;
+      const int m0 = m_tile(args, t / nt, mt) * TM + rank * BM, n0 = (t % nt) * bn;
       const int row0 = m0 + q * 32;
       for (int c = 0; c < bn; c += 32) {
         if (n0 + c >= N) break;
@@ -727,7 +731,7 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
           const int col = n0 + c + lane;
           const bool cok = col < N;
           const float bv = (cok && args.bias) ? args.bias[col] : 0.0f;
-          float* out = static_cast<float*>(args.out) + (t / mn_tiles) * args.split_stride;
+          float* out = static_cast<float*>(args.out);
 #pragma unroll 8
           for (int i = 0; i < 32; ++i) {
             const int row = row0 + i;
@@ -903,6 +907,7 @@ cudaError_t gemm_init_attributes() {
   SET_ATTR(EPI_BIAS_GELU_BF16)
   SET_ATTR(EPI_BIAS_RESID_F32)
   SET_ATTR(EPI_BIAS_ADD_F32)
+  SET_ATTR(EPI_PART_F32)
   SET_ATTR(EPI_BIAS_F32)
   SET_ATTR(EPI_BIAS_RELU_BF16)
   SET_ATTR(EPI_BIAS_RESID_RELU_BF16)
@@ -1003,7 +1008,7 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
   *p = GemmPlan{};
   if (epi == EPI_BIAS_RESID_F32) epi = EPI_BIAS_ADD_F32;  // the residual is the output itself
   const bool resid16 = is_resid16(epi);
-  const bool f32_out = epi == EPI_BIAS_ADD_F32;
+  const bool f32_out = epi == EPI_BIAS_ADD_F32 || epi == EPI_PART_F32;
   const bool tma_out = epi != EPI_BIAS_F32;
   GemmArgs& a = p->args;
   a.f16 = (epi == EPI_BIAS_RELU_F16 || epi == EPI_BIAS_F16 || epi == EPI_BIAS_RESID_RELU_F16) ? 1 : 0;
@@ -1096,8 +1101,16 @@ elasto_status gemm_plan_split_resid(GemmPlan* p, const bf16* A, int M_cap, const
   if (best_bn == 0 || !part || N % 4 != 0 || ldo % 4 != 0)
     return gemm_plan(p, A, M_cap, W, N, K, bias, out, ldo, EPI_BIAS_RESID_F32, status, W_lo, M_rows, ldw);
   elasto_status st =
-      gemm_plan(p, A, M_cap, W, N, K, nullptr, part, N, EPI_BIAS_F32, status, W_lo, rows, ldw, best_bn);
+      gemm_plan(p, A, M_cap, W, N, K, nullptr, part, N, EPI_PART_F32, status, W_lo, rows, ldw, best_bn);
   if (st != ELASTO_OK) return st;
+  // [split][row][N], rows past `rows` of a tile clipped
+  const uint64_t pd[3] = {uint64_t(N), uint64_t(rows), uint64_t(best_ks)};
+  const uint64_t ps[2] = {uint64_t(N) * 4, uint64_t(rows) * N * 4};
+  const uint32_t pb[3] = {32u, 32u, 1u};
+  if (!encode_tmap_plain(&p->tmC, part, 3, pd, ps, pb, true, true)) {
+    set_error("gemm_plan_split_resid: tensor map (alignment or size)");
+    return ELASTO_ERR_UNSUPPORTED;
+  }
   p->args.ksplit = best_ks;
   p->args.split_stride = static_cast<long long>(rows) * N;
   p->rbias = bias;
@@ -1330,6 +1343,7 @@ cudaError_t gemm_launch_main(const GemmPlan& p, int M, cudaStream_t s) {
     CASE_PAIR(EPI_BIAS_RESID_F32)
     CASE_PAIR(EPI_BIAS_ADD_F32)
     CASE(EPI_BIAS_F32)
+    CASE(EPI_PART_F32)
     CASE_PAIR(EPI_BIAS_RELU_BF16)
     CASE(EPI_BIAS_RESID_RELU_BF16)
     CASE_PAIR(EPI_BIAS_RELU_F16)
