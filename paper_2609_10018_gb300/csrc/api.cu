@@ -64,9 +64,11 @@ cudaError_t ensure_kernel_attributes() {
 }
 
 elasto_status check_device() {
+  static std::atomic<bool> fits[64];  // devices found to be sm_103 with the kernels' attributes set
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if (dev >= 0 && dev < 64 && fits[dev].load(std::memory_order_acquire)) return ELASTO_OK;
   int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
@@ -78,6 +80,7 @@ elasto_status check_device() {
   }
   e = ensure_kernel_attributes();
   if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+  fits[dev].store(true, std::memory_order_release);
   return ELASTO_OK;
 }
 
@@ -401,8 +404,10 @@ elasto_status vit_create(const elasto_model_desc* d, const elasto_weights* wts, 
   // k images' worth (k * n >= n + 128 rows) serve every batch
   h->addend_rows = (1 + (128 + n - 1) / n) * n;
   const size_t o_tok = bump.take(size_t(h->addend_rows) * D * 4, "patch token addend");
-  // split-K partial sums of the one-image FC2 (kSplitMax x n x D fp32)
-  const size_t o_part = bump.take(size_t(kSplitMax) * n * D * 4, "split-K partial sums");
+  // split-K partial sums of the small-batch out-projections and FC2s (and of
+  // the one-launch forward: up to kSplitMax of n x D)
+  const size_t part_floats = std::max(split_part_floats(num_sms()), size_t(kSplitMax) * n * D);
+  const size_t o_part = bump.take(part_floats * 4, "split-K partial sums");
   const size_t img_bytes = size_t(Bm) * d->img_h * d->img_w * d->img_c * dtype_size(d->weight_dtype);
   const size_t o_img = bump.take(img_bytes, "image staging"), o_logit = bump.take(size_t(Bm) * C * 4, "logit staging");
   const size_t o_status = bump.take(64, "status word");
@@ -830,11 +835,12 @@ elasto_status vit_create(const elasto_model_desc* d, const elasto_weights* wts, 
         vm.launches += 2;
       }
       st = plan_set(lp.proj, [&](GemmPlan& gp, int rows) {
-        // one image: the reduction split over idle SMs, and LN2 computed by
+        // few rows: the reduction split over idle SMs, and LN2 computed by
         // the launch that adds the partial sums
-        if (rows <= n) {
+        if (rows <= 8 * n) {
           const elasto_status r = gemm_plan_split_resid(&gp, h->O, Mcap, lp.proj_w, Dm, lp.w, em.proj_b[l], h->X, Dm,
-                                                        h->status, lp.proj_w_lo, rows, lp.ld_proj, h->splitk_part);
+                                                        h->status, lp.proj_w_lo, rows, lp.ld_proj, h->splitk_part,
+                                                        part_floats);
           if (r == ELASTO_OK) gemm_split_fuse_layernorm(&gp, em.ln2_w[l], em.ln2_b[l], h->Y, em.d);
           return r;
         }
@@ -851,11 +857,12 @@ elasto_status vit_create(const elasto_model_desc* d, const elasto_weights* wts, 
         vm.launches += 1;
       }
       st = plan_set(lp.fc2, [&](GemmPlan& gp, int rows) {
-        // one image: the 3072-long reduction split over the idle SMs, and
-        // the next layer's LN1 computed by the launch that adds the partials
-        if (rows <= n) {
+        // few rows: the long reduction split over the idle SMs, and the next
+        // layer's LN1 computed by the launch that adds the partials
+        if (rows <= 8 * n) {
           const elasto_status r = gemm_plan_split_resid(&gp, h->H, Mcap, lp.fc2_w, Dm, lp.f_pad, em.fc2_b[l], h->X,
-                                                        Dm, h->status, lp.fc2_w_lo, rows, lp.ld_fc2, h->splitk_part);
+                                                        Dm, h->status, lp.fc2_w_lo, rows, lp.ld_fc2, h->splitk_part,
+                                                        part_floats);
           if (r == ELASTO_OK && l + 1 < L) gemm_split_fuse_layernorm(&gp, em.ln1_w[l + 1], em.ln1_b[l + 1], h->Y, em.d);
           return r;
         }

@@ -184,14 +184,16 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
 // EPI_BIAS_RESID_F32 (out[r, :] += A W^T + bias) for at most M_rows rows with
 // the reduction split over up to kSplitMax CTAs per tile when the tiles alone
 // would leave most SMs idle (a long K on a few rows: FC2 at batch 1). The
-// partial sums go to part [ksplit, M_rows, N] fp32 (kSplitMax * M_rows * N
-// floats), then a second launch adds them in split order with the bias to
+// partial sums go to part [ksplit, M_rows, N] fp32 (part_floats of them at
+// most), then a second launch adds them in split order with the bias to
 // out: deterministic. Falls back to the single-pass plan when splitting
 // would not spread the work.
 constexpr int kSplitMax = 8;
+// Enough for any split plan of the M tiles x N tiles x splits <= SMs it makes.
+inline size_t split_part_floats(int sms) { return static_cast<size_t>(sms) * 128 * 64; }
 elasto_status gemm_plan_split_resid(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, int N, int K,
                                     const float* bias, float* out, int ldo, int* status, const bf16* W_lo, int M_rows,
-                                    int ldw, float* part);
+                                    int ldw, float* part, size_t part_floats);
 // For a split plan (does nothing otherwise, and says so by returning false):
 // the launch that adds the partial sums also writes y = LayerNorm(out row)
 // (gamma g, beta b, statistics over the first d_true of the N channels, the

@@ -1080,7 +1080,7 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
 
 elasto_status gemm_plan_split_resid(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, int N, int K,
                                     const float* bias, float* out, int ldo, int* status, const bf16* W_lo, int M_rows,
-                                    int ldw, float* part) {
+                                    int ldw, float* part, size_t part_floats) {
   const int sms = num_sms() > 0 ? num_sms() : 148;
   const int rows = (M_rows > 0 && M_rows < M_cap) ? M_rows : M_cap;
   const int mt = (rows + BM - 1) / BM, nk = (K + BK - 1) / BK;
@@ -1090,7 +1090,7 @@ elasto_status gemm_plan_split_resid(GemmPlan* p, const bf16* A, int M_cap, const
   for (int bn : {64, 32}) {
     const int tiles = mt * ((N + bn - 1) / bn);
     const int ks = std::min({kSplitMax, sms / std::max(tiles, 1), nk / 4});
-    if (ks < 2) continue;
+    if (ks < 2 || static_cast<size_t>(ks) * rows * N > part_floats) continue;
     const int kb = (nk + ks - 1) / ks;
     if (kb < best_kb) {
       best_kb = kb;
@@ -1098,6 +1098,10 @@ elasto_status gemm_plan_split_resid(GemmPlan* p, const bf16* A, int M_cap, const
       best_ks = ks;
     }
   }
+  // past one image's rows the partial sums cost more: worth it from 16 k-blocks
+  // (of one weight plane) saved (ViT-B 3 images, FC2 48 -> 24: 572 -> 525 us a
+  // forward; ViT-S 4 images, FC2 18 -> 6, lost: 384 -> 396)
+  if (rows > 256 && (nk - best_kb) * (W_lo ? 2 : 1) < 16) best_bn = 0;
   if (best_bn == 0 || !part || N % 4 != 0 || ldo % 4 != 0)
     return gemm_plan(p, A, M_cap, W, N, K, bias, out, ldo, EPI_BIAS_RESID_F32, status, W_lo, M_rows, ldw);
   elasto_status st =
