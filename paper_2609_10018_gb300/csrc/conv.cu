@@ -22,13 +22,13 @@
 // into 16-byte stores of whole pixels), warp 10 filter producer. Every mbarrier
 // wait is bounded; a timeout records ELASTO_ERR_TIMEOUT.
 //
-// What bounds it: the tensor core takes 64 clocks for a 128-row K = 16 step of
-// up to 128 channels (its input rows arrive at 64 B a clock), so 64 channels
-// run at half the rate of 128. Back-to-back calls, box per tap -> here: 128
-// images of 56 x 56 x 64 -> 64 channels 67.5 -> 35.9 us (62 clocks a step
-// inside), 28 x 28 x 128 -> 128 35.3 -> 20.3 us (1.46 PFLOP/s), 14 x 14 x 192 ->
-// 192 20.6 -> 17.0 us, 16 images of 56 x 56 x 64 12.2 -> 8.4 us. 7 x 7 images
-// (49 of 128 rows) and at most 16 channels stay with the box per tap.
+// What bounds it: the MMAs, and issuing them: the taps are unrolled, with 32-bit
+// descriptor sums (tc_mma_pair_warp_lo), for 3 x 3 and the stem's 1 x 4.
+// Back-to-back calls, box per tap -> here: 128 images of 56 x 56 x 64 -> 64
+// channels 67.5 -> 27.5 us (35.9 with the taps in a loop), 28 x 28 x 128 -> 128
+// 35.3 -> 20.5 us (1.45 PFLOP/s), 28 x 28 x 96 -> 96 35.5 -> 16.8, 14 x 14 x 192 ->
+// 192 20.5 -> 17.0, 16 images of 56 x 56 x 64 12.3 -> 7.6 us. 7 x 7 images (49 of
+// 128 rows) and at most 16 channels stay with the box per tap.
 #include <algorithm>
 
 #include "common.h"
@@ -57,7 +57,8 @@ __device__ __forceinline__ Block block_at(const HaloArgs& a, int i) {
   return {r / a.nby, (r % a.nby) * a.bh, (i - r * a.nbx) * a.bw};
 }
 
-template <bool RELU>
+// TX x TY taps known at compile time (3 x 3, and the stem's 1 x 4), or 0.
+template <bool RELU, int TX, int TY>
 __global__ void __launch_bounds__(THREADS, 1)
     conv_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                      const HaloArgs a) {
@@ -199,6 +200,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     // ------------------------------------------------------------ MMA issuer
     if (leader) {
       const uint32_t idesc = idesc_16_f32(2 * ROWS, a.bn, true);
+      const uint32_t a_base = sdesc_lo(smem_addr(sA), 16), b_base = sdesc_lo(smem_addr(sB), 16);
+      const uint32_t hi = sdesc_sw128_hi(1024), b_units = b_bytes >> 4;
       int as = 0, bs = 0, local = 0;
       uint32_t aph = 0, bph = 0;
       bool ok = t0 >= tiles || !a.b_resident || mbar_wait_warp(&b_full[0], 0);
@@ -217,31 +220,50 @@ __global__ void __launch_bounds__(THREADS, 1)
             break;
           }
           tc_fence_after();
-          uint64_t row = sdesc_sw128(smem_addr(sA + as * a.a_stage), 16, 1024);  // tap (ky, 0): +8 per halo row
-          int tap = 0;
-          for (int ky = 0; ky < a.taps_y && ok; ++ky, row += 8 * a.wp)
-            for (int kx = 0; kx < a.taps_x; ++kx, ++tap) {
-              if (!a.b_resident) {
-                if (!mbar_wait_warp(&b_full[bs], bph)) {
-                  ok = false;
-                  break;
-                }
-                tc_fence_after();
-              }
-              const uint64_t da = row + 8 * kx;
-              const uint64_t db =
-                  sdesc_sw128(smem_addr(sB + (a.b_resident ? tap * a.cgroups + g : bs) * b_bytes), 16, 1024);
+          // tap (ky, kx) starts 8 * (ky * wp + kx) 16-byte units after the halo
+          const uint32_t a_lo = a_base + as * (a.a_stage >> 4), wp8 = 8u * a.wp;
+          auto tap_mma = [&](uint32_t lo, uint32_t b_lo, uint32_t accumulate) {
 #pragma unroll
-              for (int k = 0; k < 4; ++k) tc_mma_pair_warp(d, da + 2 * k, db + 2 * k, idesc, (g | tap | k) != 0);
-              issued = true;
-              if (!a.b_resident) {
-                tc_commit_pair_multicast_warp(&b_empty[bs], 0x3);
-                if (++bs == a.b_stages) {
-                  bs = 0;
-                  bph ^= 1;
-                }
-              }
+            for (uint32_t k = 0; k < 4; ++k)
+              tc_mma_pair_warp_lo(d, lo + 2 * k, b_lo + 2 * k, hi, idesc, k > 0 ? 1u : accumulate);
+          };
+          auto streamed_tap = [&](uint32_t lo, uint32_t accumulate) -> bool {
+            if (!mbar_wait_warp(&b_full[bs], bph)) return false;
+            tc_fence_after();
+            tap_mma(lo, b_base + bs * b_units, accumulate);
+            tc_commit_pair_multicast_warp(&b_empty[bs], 0x3);
+            if (++bs == a.b_stages) {
+              bs = 0;
+              bph ^= 1;
             }
+            return true;
+          };
+          if constexpr (TX > 0) {  // unrolled: issuing has to keep up with the MMAs
+            if (a.b_resident) {
+#pragma unroll
+              for (int ky = 0; ky < TY; ++ky)
+#pragma unroll
+                for (int kx = 0; kx < TX; ++kx)
+                  tap_mma(a_lo + ky * wp8 + 8 * kx, b_base + ((ky * TX + kx) * a.cgroups + g) * b_units,
+                          ky + kx > 0 ? 1u : g != 0);
+            } else {
+#pragma unroll
+              for (int ky = 0; ky < TY; ++ky)
+#pragma unroll
+                for (int kx = 0; kx < TX; ++kx)
+                  if (ok) ok = streamed_tap(a_lo + ky * wp8 + 8 * kx, ky + kx > 0 ? 1u : g != 0);
+            }
+          } else {
+            for (int ky = 0; ky < a.taps_y && ok; ++ky)
+              for (int kx = 0; kx < a.taps_x && ok; ++kx) {
+                const uint32_t lo = a_lo + ky * wp8 + 8 * kx;
+                if (a.b_resident)
+                  tap_mma(lo, b_base + ((ky * a.taps_x + kx) * a.cgroups + g) * b_units, (g | ky | kx) != 0);
+                else
+                  ok = streamed_tap(lo, (g | ky | kx) != 0);
+              }
+          }
+          issued = true;
           tc_commit_pair_multicast_warp(&a_empty[as], 0x3);
           if (++as == a.a_stages) {
             as = 0;
@@ -361,15 +383,26 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
+using HaloKernel = void (*)(CUtensorMap, CUtensorMap, HaloArgs);
+HaloKernel halo_kernel(bool relu, int taps_x, int taps_y) {
+  if (taps_x == 3 && taps_y == 3) return relu ? conv_halo_kernel<true, 3, 3> : conv_halo_kernel<false, 3, 3>;
+  if (taps_x == 1 && taps_y == 4) return relu ? conv_halo_kernel<true, 1, 4> : conv_halo_kernel<false, 1, 4>;
+  return relu ? conv_halo_kernel<true, 0, 0> : conv_halo_kernel<false, 0, 0>;
+}
+
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 }  // namespace
 
 cudaError_t halo_init_attributes() {
   const int bytes = static_cast<int>(SMEM_BYTES);
-  cudaError_t e = cudaFuncSetAttribute(conv_halo_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(conv_halo_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaSuccess;
+  for (int relu = 0; relu < 2; ++relu)
+    for (int t = 0; t < 3; ++t)
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(halo_kernel(relu != 0, t == 2 ? 1 : 3 * t, t == 2 ? 4 : 3 * t)),
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
 }
 
 bool halo_layout(HaloArgs* a, int batch, int Ho, int Wo, int taps_x, int taps_y, int cgroups, int pad, int N, int sms,
@@ -430,8 +463,8 @@ bool halo_layout(HaloArgs* a, int batch, int Ho, int Wo, int taps_x, int taps_y,
       b.b_stages = std::min((pool - b.a_stages * b.a_stage) / b_bytes, MAX_B);
       if (pool < b.a_stages * b.a_stage || b.b_stages < 3) continue;
     }
-    // a 128-row K = 16 step takes 64 clocks up to 128 channels; a filter wait per k-block adds ~130
-    const double mma = (4 * std::max(0.5 * b.bn, 64.0) + (b.b_resident ? 0 : 130)) / 1.9;
+    // a 128-row K = 16 step takes bn / 2 clocks, 45 at least; a filter wait per k-block adds ~130
+    const double mma = (4 * std::max(0.5 * b.bn, 45.0) + (b.b_resident ? 0 : 130)) / 1.9;
     const double load = (b.a_tx / (taps_x * taps_y) + (b.b_resident ? 0 : b_bytes)) / 126.0;
     const long tiles = (best_blocks * batch + 1) / 2 * nt, waves = (tiles + units - 1) / units;
     const double epilogue = 500.0 + 6.0 * b.bn;
@@ -475,8 +508,7 @@ cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return p.epi == EPI_BIAS_RELU_F16 ? cudaLaunchKernelEx(&cfg, conv_halo_kernel<true>, p.tmA, p.tmB, a)
-                                    : cudaLaunchKernelEx(&cfg, conv_halo_kernel<false>, p.tmA, p.tmB, a);
+  return cudaLaunchKernelEx(&cfg, halo_kernel(p.epi == EPI_BIAS_RELU_F16, a.taps_x, a.taps_y), p.tmA, p.tmB, a);
 }
 
 }  // namespace elasto

@@ -247,7 +247,7 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 // The same, called by a whole converged warp in which one elected thread
 // issues. With warp-uniform control flow around them (mbar_wait_warp, a warp
 // number from __shfl_sync) their operands stay in warp-wide registers: an MMA
-// issues every ~60 clocks (64 is what a 128-row K = 16 step takes), 70 from a
+// issues every ~60 clocks (a 256-column K = 16 step takes 103 to 128), 70 from a
 // branch of one elected thread and 115 from a branch on a lane number.
 __device__ __forceinline__ void tc_mma_warp(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                             uint32_t accumulate) {
@@ -394,6 +394,27 @@ __device__ __forceinline__ void tc_mma_pair_warp(uint32_t d_tmem, uint64_t adesc
       " @q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+// The same with the descriptors' 32-bit halves apart: only the low one (the
+// start address) differs between the tiles of a loop, and 32-bit sums of uniform
+// values stay in warp-wide registers. In unrolled code an MMA then issues
+// faster than a 128-row, 64-column, K = 16 step runs (~45 clocks; 62 with
+// 64-bit sums); wider tiles and the GEMM's loop gained nothing from it.
+__device__ __forceinline__ void tc_mma_pair_warp_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
+                                                    uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b64 da, db;\n elect.sync _|q, 0xffffffff;\n setp.ne.b32 p, %5, 0;\n"
+      " mov.b64 da, {%1, %3};\n mov.b64 db, {%2, %3};\n"
+      " @q tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Halves of sdesc_sw128(saddr, lbo, sbo).
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr, uint32_t lbo_bytes) {
+  return ((saddr & 0x3FFFFu) >> 4) | (lbo_bytes >> 4) << 16;
+}
+__device__ __forceinline__ constexpr uint32_t sdesc_sw128_hi(uint32_t sbo_bytes) {
+  return (sbo_bytes >> 4) | 1u << 14 | 2u << 29;
 }
 __device__ __forceinline__ void tc_commit_pair_multicast_warp(uint64_t* bar, uint16_t mask) {
   asm volatile(
