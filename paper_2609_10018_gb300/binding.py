@@ -202,8 +202,6 @@ def weights_struct(keep: _Keep, tensors: Sequence[np.ndarray]) -> Weights:
 # ----------------------------------------------------------------------------
 # C-ABI calls (same names)
 # ----------------------------------------------------------------------------
-# The calls of a request path skip two Python calls where they can: a small op
-# is bound by its host side (7 us with the caller's, 3 of it in the library).
 
 def elasto_create(desc: ModelDesc, tensors: Sequence[np.ndarray], mode_tables, n_modes: int | None = None,
                   keep: _Keep | None = None) -> int:
@@ -227,9 +225,7 @@ def elasto_get_mode(h: int) -> int:
 
 
 def elasto_forward(h: int, stream: int, images_ptr: int, batch: int, logits_ptr: int) -> None:
-    st = (_lib or lib()).elasto_forward(h, stream, images_ptr, batch, logits_ptr)
-    if st:
-        _check(st, "elasto_forward")
+    _check(lib().elasto_forward(h, stream, images_ptr, batch, logits_ptr), "elasto_forward")
 
 
 def elasto_forward_noalloc(h: int, stream: int, images_ptr: int, batch: int, logits_ptr: int) -> None:
@@ -376,33 +372,24 @@ def saliency_tables_vit(cfg, weights, names=None, embed_widths=None):
 
 
 def elasto_op_gemm(stream, A, W, bias, out, resid, M, N, K, epilogue, status=0) -> None:
-    st = (_lib or lib()).elasto_op_gemm(stream, A, W, bias, out, resid, M, N, K, epilogue, status)
-    if st:
-        _check(st, "elasto_op_gemm")
+    _check(lib().elasto_op_gemm(stream, A, W, bias, out, resid, M, N, K, epilogue, status), "elasto_op_gemm")
 
 
 def elasto_op_conv2d(stream, x, B, H, W, C, w, N, k, stride, pad, bias, relu, out, status=0) -> None:
-    st = (_lib or lib()).elasto_op_conv2d(stream, x, B, H, W, C, w, N, k, stride, pad, bias, int(relu), out, status)
-    if st:
-        _check(st, "elasto_op_conv2d")
+    _check(lib().elasto_op_conv2d(stream, x, B, H, W, C, w, N, k, stride, pad, bias, int(relu), out, status),
+           "elasto_op_conv2d")
 
 
 def elasto_op_layernorm(stream, x, gamma, beta, y, rows, d) -> None:
-    st = (_lib or lib()).elasto_op_layernorm(stream, x, gamma, beta, y, rows, d)
-    if st:
-        _check(st, "elasto_op_layernorm")
+    _check(lib().elasto_op_layernorm(stream, x, gamma, beta, y, rows, d), "elasto_op_layernorm")
 
 
 def elasto_op_softmax(stream, x, y, rows, cols) -> None:
-    st = (_lib or lib()).elasto_op_softmax(stream, x, y, rows, cols)
-    if st:
-        _check(st, "elasto_op_softmax")
+    _check(lib().elasto_op_softmax(stream, x, y, rows, cols), "elasto_op_softmax")
 
 
 def elasto_op_attention(stream, qkv, out, batch, n, heads, status=0) -> None:
-    st = (_lib or lib()).elasto_op_attention(stream, qkv, out, batch, n, heads, status)
-    if st:
-        _check(st, "elasto_op_attention")
+    _check(lib().elasto_op_attention(stream, qkv, out, batch, n, heads, status), "elasto_op_attention")
 
 
 def elasto_op_bounded_wait(stream, armed: bool, status, elapsed_ns) -> None:
