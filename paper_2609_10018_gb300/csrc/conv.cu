@@ -23,12 +23,18 @@
 // wait is bounded; a timeout records ELASTO_ERR_TIMEOUT.
 //
 // What bounds it: the MMAs, and issuing them: the taps are unrolled, with 32-bit
-// descriptor sums (tc_mma_pair_warp_lo), for 3 x 3 and the stem's 1 x 4.
+// descriptor sums (tc_mma_pair_warp_lo), for 3 x 3 and the stem's 1 x 4; below 64
+// output channels and in the stem the epilogue, whose tile coordinates advance by
+// additions (TileWalk; 128 images of 56 x 56 x 32 27.0 -> 24.3 us, the stem 81 ->
+// 70). Tried there without gain: a third group of epilogue warps (stem 73), four
+// accumulators instead of two (72).
 // Back-to-back calls, box per tap -> here: 128 images of 56 x 56 x 64 -> 64
-// channels 67.5 -> 27.5 us (35.9 with the taps in a loop), 28 x 28 x 128 -> 128
+// channels 67.5 -> 26.5 us (35.9 with the taps in a loop), 28 x 28 x 128 -> 128
 // 35.3 -> 20.5 us (1.45 PFLOP/s), 28 x 28 x 96 -> 96 35.5 -> 16.8, 14 x 14 x 192 ->
-// 192 20.5 -> 17.0, 16 images of 56 x 56 x 64 12.3 -> 7.6 us. 7 x 7 images (49 of
-// 128 rows) and at most 16 channels stay with the box per tap.
+// 192 20.5 -> 17.0, 16 images of 56 x 56 x 64 12.3 -> 7.5 us. 7 x 7 images (49 of
+// 128 rows) and at most 16 channels stay with the box per tap. So do strides: the
+// four parity tiles of a 3 x 3 of stride 2 hold one to four taps each (100 images
+// of 28 x 28 x 192 at stride 2: 23.7 us on such tiles, 19.0 with a box per tap).
 #include <algorithm>
 
 #include "common.h"
@@ -49,13 +55,53 @@ constexpr int BARS = 2 * MAX_A + 2 * MAX_B + 6;  // mbarriers: rings, tfull, tem
 static_assert(BARS * 8 % 16 == 0 && BARS * 8 + EPI_WARPS * 128 + 4 <= 2048, "barriers and bias");
 static_assert(SMEM_BYTES <= 232448, "shared memory");
 
-struct Block {
-  int b, oy, ox;  // image, first output row and column
+// The tiles a CTA works on, in order: N tile n and this CTA's pixel block
+// (column x, row y of image b) of tile t0, t0 + step, ... Advanced by additions
+// with carries: the divisions, one after another, are a large part of a narrow
+// tile's time otherwise.
+struct TileWalk {
+  struct Pos {
+    int x, y, b;
+  };
+  int n;
+  Pos k;
+  int nt, nbx, nby, dn;
+  Pos d, pair;  // blocks between two tiles, and in a pair
+
+  __device__ __forceinline__ Pos split(int i) const {
+    const int r = i / nbx;
+    return {i - r * nbx, r % nby, r / nby};
+  }
+  __device__ __forceinline__ void add(const Pos& v) {
+    k.x += v.x;
+    k.y += v.y;
+    k.b += v.b;
+    if (k.x >= nbx) {
+      k.x -= nbx;
+      ++k.y;
+    }
+    if (k.y >= nby) {
+      k.y -= nby;
+      ++k.b;
+    }
+  }
+  __device__ __forceinline__ TileWalk(const HaloArgs& a, int nt_, int t0, int step, int rank)
+      : nt(nt_), nbx(a.nbx), nby(a.nby) {
+    n = t0 % nt;
+    dn = step % nt;
+    k = split(t0 / nt * 2 + rank);
+    d = split(step / nt * 2);
+    pair = split(2);
+  }
+  __device__ __forceinline__ void next() {
+    add(d);
+    n += dn;
+    if (n >= nt) {
+      n -= nt;
+      add(pair);
+    }
+  }
 };
-__device__ __forceinline__ Block block_at(const HaloArgs& a, int i) {
-  const int r = i / a.nbx;
-  return {r / a.nby, (r % a.nby) * a.bh, (i - r * a.nbx) * a.bw};
-}
 
 // TX x TY taps known at compile time (3 x 3, and the stem's 1 x 4), or 0.
 template <bool RELU, int TX, int TY>
@@ -137,17 +183,17 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t ph = 0;
       bool ok = true;
       long issued = 0;
-      for (int t = t0; t < tiles && ok; t += step) {
+      TileWalk w(a, nt, t0, step, rank);
+      for (int t = t0; t < tiles && ok; t += step, w.next()) {
         // (the last pair's second block may not exist: b = batch, all read as zero or never stored)
-        const Block k = block_at(a, (t / nt) * 2 + rank);
         for (int g = 0; g < a.cgroups; ++g) {
           if (!mbar_wait(&a_empty[s], ph ^ 1)) {
             ok = false;
             break;
           }
           if (leader) mbar_expect_tx(&a_full[s], 2u * a.a_tx);
-          tma_load_4d_pair(sA + s * a.a_stage, &tmX, cluster_map(smem_addr(&a_full[s]), 0), g * 64, k.ox - a.pad,
-                           k.oy - a.pad, k.b);
+          tma_load_4d_pair(sA + s * a.a_stage, &tmX, cluster_map(smem_addr(&a_full[s]), 0), g * 64, w.k.x * a.bw - a.pad,
+                           w.k.y * a.bh - a.pad, w.k.b);
           ++issued;
           if (++s == a.a_stages) {
             s = 0;
@@ -170,8 +216,10 @@ __global__ void __launch_bounds__(THREADS, 1)
       uint32_t ph = 0;
       bool ok = true;
       long issued = 0;
-      for (int t = t0; t < tiles && ok; t += step) {
-        const int row = (t % nt) * a.bn + rank * half;
+      int n = t0 % nt;
+      const int dn = step % nt;
+      for (int t = t0; t < tiles && ok; t += step, n = n + dn >= nt ? n + dn - nt : n + dn) {
+        const int row = n * a.bn + rank * half;
         for (int g = 0; g < a.cgroups && ok; ++g)
           for (int tap = 0; tap < taps; ++tap) {
             if (!mbar_wait(&b_empty[s], ph ^ 1)) {
@@ -285,18 +333,27 @@ __global__ void __launch_bounds__(THREADS, 1)
     float* sb = sbias + 32 * ew;
     // this lane's part of the stores: 16 bytes (8 channels) of eight pixels
     const int piece = lane & 7;
-    int rel[8], pos[8];  // pixel offset from the block's first, (y << 16 | x); pos < 0: not an output
+    uint32_t off[8], keep = 0;  // 16-byte units from the block's first pixel; bit i: row i is an output pixel
+    int pos[8];                 // y << 16 | x
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int r = q * 32 + i * 4 + (lane >> 3), y = r / a.wp, x = r - y * a.wp;
-      rel[i] = y * a.Wo + x;
-      pos[i] = y < a.bh && x < a.bw ? (y << 16 | x) : -1;
+      off[i] = static_cast<uint32_t>(y * a.Wo + x) * static_cast<uint32_t>(a.ldo / 8);
+      pos[i] = y << 16 | x;
+      keep |= (y < a.bh && x < a.bw ? 1u : 0u) << i;
+    }
+    const bool one = nt == 1;  // N <= 256: the whole bias is kept in sbias
+    if (one) {
+      const int c = static_cast<int>(threadIdx.x) - 64;
+      sbias[c] = a.bias && c < a.N ? __ldg(a.bias + c) : 0.0f;
+      named_bar_sync(1, 32 * EPI_WARPS);
     }
     const uint32_t row_tm = tmem + (static_cast<uint32_t>(q * 32) << 16);
     int local = 0, before = 0;
     bool ok = true;
-    for (int t = t0; t < tiles; t += step, ++local) {
-      const int acc = local & 1, bi = (t / nt) * 2 + rank, n0 = (t % nt) * a.bn;
+    TileWalk w(a, nt, t0, step, rank);
+    for (int t = t0; t < tiles; t += step, ++local, w.next()) {
+      const int acc = local & 1, n0 = w.n * a.bn;
       const int width = min(a.bn, a.N - n0), chunks = (width + 63) / 64;
       int c = grp ^ before;
       before ^= chunks & 1;
@@ -308,7 +365,15 @@ __global__ void __launch_bounds__(THREADS, 1)
           nb[h] = a.bias && k < width ? __ldg(a.bias + n0 + k) : 0.0f;
         }
       };
-      bias_of(c);
+      if (!one) bias_of(c);
+      const int oy = w.k.y * a.bh, ox = w.k.x * a.bw;
+      uint32_t outs = keep;  // of an edge block less
+      if (oy + a.bh > a.Ho || ox + a.bw > a.Wo || w.k.b >= a.batch) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (oy + (pos[i] >> 16) >= a.Ho || ox + (pos[i] & 0xffff) >= a.Wo || w.k.b >= a.batch) outs &= ~(1u << i);
+      }
+      __half* first = static_cast<__half*>(a.out) + ((static_cast<size_t>(w.k.b) * a.Ho + oy) * a.Wo + ox) * a.ldo + n0;
       ok = __all_sync(0xffffffffu, mbar_wait(&tfull[acc], static_cast<uint32_t>((local >> 1) & 1)));
       if (!ok) break;
       tc_fence_after();
@@ -318,37 +383,40 @@ __global__ void __launch_bounds__(THREADS, 1)
         if (lane == 0) mbar_arrive_cluster(cluster_map(smem_addr(&tempty[acc]), 0));
       };
       if (c >= chunks) release();
-      const Block k = block_at(a, bi);
       for (; c < chunks; c += 2) {
         uint32_t v[2][32];
         tmem_ld_32x32b_x32(row_tm + acc * ACC_COLS + c * 64, v[0]);
         tmem_ld_32x32b_x32(row_tm + acc * ACC_COLS + c * 64 + 32, v[1]);
         const float bl[2] = {nb[0], nb[1]};
-        if (c + 2 < chunks) bias_of(c + 2);
+        if (!one && c + 2 < chunks) bias_of(c + 2);
         tmem_ld_wait();
         if (c + 2 >= chunks) release();
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          __syncwarp();
-          sb[lane] = bl[h];
-          __syncwarp();
+          const float* bias = sbias + c * 64 + 32 * h;
+          if (!one) {
+            bias = sb;
+            __syncwarp();
+            sb[lane] = bl[h];
+            __syncwarp();
+          }
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             uint32_t ow[4];
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
-              const float4 b4 = reinterpret_cast<const float4*>(sb)[2 * j + i];
+              const float4 b4 = reinterpret_cast<const float4*>(bias)[2 * j + i];
               float2 lo = add2(make_float2(__uint_as_float(v[h][8 * j + 4 * i]), __uint_as_float(v[h][8 * j + 4 * i + 1])),
                                make_float2(b4.x, b4.y));
               float2 hi =
                   add2(make_float2(__uint_as_float(v[h][8 * j + 4 * i + 2]), __uint_as_float(v[h][8 * j + 4 * i + 3])),
                        make_float2(b4.z, b4.w));
-              if (RELU) {
-                lo = make_float2(fmaxf(lo.x, 0.0f), fmaxf(lo.y, 0.0f));
-                hi = make_float2(fmaxf(hi.x, 0.0f), fmaxf(hi.y, 0.0f));
-              }
               ow[2 * i] = pack_f16x2(lo.x, lo.y);
               ow[2 * i + 1] = pack_f16x2(hi.x, hi.y);
+              if (RELU) {  // rounding keeps the sign, so the maximum can follow it
+                ow[2 * i] = relu_f16x2(ow[2 * i]);
+                ow[2 * i + 1] = relu_f16x2(ow[2 * i + 1]);
+              }
             }
             *reinterpret_cast<uint4*>(buf + lane * 128 + (((4 * h + j) ^ (lane & 7)) << 4)) =
                 make_uint4(ow[0], ow[1], ow[2], ow[3]);
@@ -356,16 +424,12 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         __syncwarp();
         const int col = c * 64 + piece * 8;
-        if (bi < blocks && col < width) {
-          uint4* dst = reinterpret_cast<uint4*>(static_cast<__half*>(a.out) +
-                                                ((static_cast<size_t>(k.b) * a.Ho + k.oy) * a.Wo + k.ox) * a.ldo + n0 +
-                                                col);
+        if (col < width) {
+          uint4* dst = reinterpret_cast<uint4*>(first + col);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const int r = i * 4 + (lane >> 3);
-            if (pos[i] >= 0 && k.oy + (pos[i] >> 16) < a.Ho && k.ox + (pos[i] & 0xffff) < a.Wo)
-              dst[static_cast<size_t>(rel[i]) * a.ldo / 8] =
-                  *reinterpret_cast<const uint4*>(buf + r * 128 + ((piece ^ (r & 7)) << 4));
+            if (outs >> i & 1) dst[off[i]] = *reinterpret_cast<const uint4*>(buf + r * 128 + ((piece ^ (r & 7)) << 4));
           }
         }
         __syncwarp();  // the staging rows are read before the next chunk writes them

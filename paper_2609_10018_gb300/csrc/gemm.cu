@@ -1200,7 +1200,8 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
   a.pair = pair ? 1 : 0;
   // halo tiles where they are estimated faster than a box per tap
   double halo = 0.0;
-  if (!k16 && stride == 1 &&
+  // (its offsets within an image are 32-bit, in 16-byte units)
+  if (!k16 && stride == 1 && static_cast<int64_t>(Ho) * Wo * ldo < (int64_t(1) << 34) &&
       halo_layout(&p->halo, B_cap, Ho, Wo, taps_x, taps / taps_x, cg, pad, N, prob.sms, &halo) &&
       halo < tile_cost(prob, a.bn, pair)) {
     p->halo.bias = bias;
