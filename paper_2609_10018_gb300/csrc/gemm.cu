@@ -74,7 +74,7 @@ constexpr int A_STAGE = BM * BK * 2;        // 16 KB
 constexpr int WBUF = 32 * 128;              // 4 KB staging piece of one epilogue warp (32 rows x 128 B)
 constexpr int CBUF = MAX_EPI_WARPS * WBUF;  // 48 KB: one staging piece for each of twelve epilogue warps
 constexpr int POOL = 224 * 1024;            // operand ring + staging pieces
-constexpr int MAX_CBUFS = 2;                // staging pieces per epilogue warp
+constexpr int MAX_CBUFS = 3;                // staging pieces per epilogue warp
 constexpr int EPI_LD = 33;                  // padded row of the transpose tile
 constexpr int EPI_TILE = 32 * EPI_LD;       // floats per epilogue warp
 constexpr int TMEM_COLS = 512;
@@ -954,7 +954,16 @@ double tile_cost(const Problem& p, int bn, bool pair) {
   if (p.conv) load = std::max(load, 280.0);  // 4-D boxes
   const double main_loop = ((p.K + BK - 1) / BK) * std::max(load, mma);
   const bool f32 = p.epi == EPI_BIAS_RESID_F32 || p.epi == EPI_BIAS_ADD_F32;
-  const double epilogue = 400.0 + bn * (f32 ? 8.0 : p.epi == EPI_BIAS_GELU_BF16 ? 9.0 : 6.0);
+  double epilogue = 400.0 + bn * (f32 ? 8.0 : p.epi == EPI_BIAS_GELU_BF16 ? 9.0 : 6.0);
+  if (is_resid16(p.epi)) {
+    // a 16-bit residual is read ahead; past the L2 it moves at the memory's pace,
+    // and later where one piece per warp is all that fits ahead (CNN block outputs,
+    // 256 -> 128 columns: 100352 x 512 x 128 43.3 -> 41.4 us, 25088 x 1024 x 256
+    // 28.2 -> 25.6, 100352 x 256 x 64 24.3 -> 22.4; 192: 6272 x 2048 x 512 17.0 -> 15.7)
+    epilogue = 550.0 + 9.0 * bn;
+    if (4.0 * p.M * p.N > 64e6) epilogue = std::max(epilogue, 200.0 + 13.0 * bn);
+    if (bn > 192) epilogue += 600.0;
+  }
   return waves * (std::max(main_loop, epilogue) + 100.0) + epilogue + (pair ? 800.0 : 0.0);
 }
 
@@ -979,14 +988,19 @@ namespace {
 
 // Splits the pool between the operand ring and the epilogue's staging pieces.
 // cbufs counts pieces per epilogue warp: with a residual read through them (its
-// fetch depth) as many as leave 3 stages, else 1.
+// fetch depth) up to two, as long as that leaves 3 stages; a 16-bit residual's
+// short tiles (one k-block) three and 2 stages (401408 x 256 x 64 in 128 columns:
+// 71.2 us, 74.6 with two pieces), its long ones need 4 stages (6272 x 2048 x 512
+// in 192 columns: 15.7 us with one piece, 16.7 with two and 3 stages).
 bool ring_layout(GemmArgs* a, int epi) {
   const int stage = a->b_stage + A_STAGE, piece = epi_warps(epi) * WBUF;
   const bool resid = epi == EPI_BIAS_RESID_F32 || is_resid16(epi);
-  for (int e = resid ? MAX_CBUFS : 1; e >= 1; --e) {
+  const bool r16 = is_resid16(epi);
+  const int most = r16 && a->K <= BK ? 3 : resid ? 2 : 1, least = r16 && a->K <= BK ? 2 : r16 && a->K > 4 * BK ? 4 : 3;
+  for (int e = most; e >= 1; --e) {
     a->cbufs = e;
     a->stages = std::min((POOL - e * piece) / stage, MAX_STAGES);
-    if (a->stages >= 3) break;
+    if (a->stages >= least) break;
   }
   return a->stages >= 2 && a->stages * stage + a->cbufs * piece <= POOL;
 }

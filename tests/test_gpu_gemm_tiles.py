@@ -1,6 +1,7 @@
 """The GEMM's tile variants at their edges, against fp64: CTA pairs at short
 reductions with ragged last rows and columns, the residual added by the store
-or read ahead, and convolutions on pairs whose last pixel block is missing."""
+or read ahead, CNN block outputs, and convolutions on pairs whose last pixel
+block is missing."""
 import numpy as np
 import pytest
 
@@ -82,3 +83,32 @@ def test_conv_pairs_match_fp64(B, S, C, N, k, stride):
     ref = np.maximum(orr.conv2d(x[pick].astype(np.float64), w.astype(np.float64), stride, k // 2) + bias, 0)
     # one f16 rounding (2^-11 relative, doubled) and fp32 accumulation
     assert np.all(np.abs(got[pick] - ref) <= 2.0 ** -10 * np.abs(ref) + 1e-4 * np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("M,N,K", [
+    (100353, 264, 64),   # one k-block a tile: the residual read three pieces ahead
+    (25089, 1032, 200),  # past the L2, 128 columns
+    (6273, 2056, 520),   # 192 columns, one piece ahead
+    (129, 72, 64),       # one wave
+])
+def test_block_output_tiles_match_fp64(M, N, K):
+    import torch
+    rng = np.random.default_rng(M + N + K)
+    A = rng.standard_normal((M, K), dtype=np.float32).astype(np.float16)
+    W = (rng.standard_normal((N, K)) * np.sqrt(2.0 / K)).astype(np.float16)
+    bias = rng.standard_normal(N).astype(np.float32)
+    R = rng.standard_normal((M, N), dtype=np.float32).astype(np.float16)
+    out = empty_dev((M, N), torch.uint16)
+    out.fill_(0x7E00)  # f16 NaN: every output must be written
+    dA, dW, db, dR = dev(A.view(np.uint16)), dev(W.view(np.uint16)), dev(bias), dev(R.view(np.uint16))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    binding.elasto_op_gemm(stream_handle(), dA.data_ptr(), dW.data_ptr(), db.data_ptr(), out.data_ptr(), dR.data_ptr(),
+                           M, N, K, binding.EPI_BIAS_RESID_RELU_F16, status.data_ptr())
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    got = out.cpu().numpy().view(np.float16)
+    assert np.all(np.isfinite(got))
+    rows = np.unique(np.concatenate([np.arange(min(M, 300)), rng.choice(M, 500), np.arange(max(0, M - 300), M)]))
+    ref = np.maximum(A[rows].astype(np.float64) @ W.astype(np.float64).T + bias + R[rows].astype(np.float64), 0)
+    # one f16 rounding (2^-11 relative, doubled) and fp32 accumulation
+    assert np.all(np.abs(got[rows].astype(np.float64) - ref) <= 2.0 ** -10 * np.abs(ref) + 1e-5 * np.max(np.abs(ref)))
