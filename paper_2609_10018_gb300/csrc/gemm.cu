@@ -988,15 +988,26 @@ namespace {
 
 // Splits the pool between the operand ring and the epilogue's staging pieces.
 // cbufs counts pieces per epilogue warp: with a residual read through them (its
-// fetch depth) up to two, as long as that leaves 3 stages; a 16-bit residual's
-// short tiles (one k-block) three and 2 stages (401408 x 256 x 64 in 128 columns:
-// 71.2 us, 74.6 with two pieces), its long ones need 4 stages (6272 x 2048 x 512
-// in 192 columns: 15.7 us with one piece, 16.7 with two and 3 stages).
+// fetch depth) as many of two as leave 3 operand stages, 5 under an fp32 residual
+// past 8 k-blocks and 4 under a 16-bit one past 4 (one piece, then two and fewer
+// stages: 50432 x 576 x 640 51.0 us, 53.6; 6272 x 2048 x 512 in 192 columns 15.7,
+// 16.7). A 16-bit residual's one-k-block tiles take three pieces and 2 stages
+// (401408 x 256 x 64 in 128 columns: 71.2 us, 74.6 with two pieces).
 bool ring_layout(GemmArgs* a, int epi) {
   const int stage = a->b_stage + A_STAGE, piece = epi_warps(epi) * WBUF;
   const bool resid = epi == EPI_BIAS_RESID_F32 || is_resid16(epi);
-  const bool r16 = is_resid16(epi);
-  const int most = r16 && a->K <= BK ? 3 : resid ? 2 : 1, least = r16 && a->K <= BK ? 2 : r16 && a->K > 4 * BK ? 4 : 3;
+  const int kb = (a->K + BK - 1) / BK;
+  int most = resid ? 2 : 1, least = 3;
+  if (is_resid16(epi)) {
+    if (kb == 1) {
+      most = MAX_CBUFS;
+      least = 2;
+    } else if (kb > 4) {
+      least = 4;
+    }
+  } else if (resid && kb > 8) {
+    least = 5;
+  }
   for (int e = most; e >= 1; --e) {
     a->cbufs = e;
     a->stages = std::min((POOL - e * piece) / stage, MAX_STAGES);
@@ -1051,13 +1062,15 @@ elasto_status gemm_plan(GemmPlan* p, const bf16* A, int M_cap, const bf16* W, in
   a.status = status;
   a.b_planes = planes;
   // Reduce-add stores move 5.1 TB/s of X, loads and stores 5.8, so X is read
-  // ahead where memory sets the pace: X past the L2 and a short reduction (50432
-  // x 768 x 192: 65 us added, 55 us read ahead; K = 1536: 92 and 100; X in the
-  // L2, 6304 x 768 x 768: 11.5 and 14.9). And on a nearly idle chip, where the
-  // read hides behind the main loop and a reduce-add completes later.
+  // ahead where memory sets the pace: X past the L2 and a short reduction. 50432 x
+  // 768: K = 192 64.5 us added, 54.7 read ahead; 576 65.9, 62.3; 768 67.4, 67.6;
+  // 1536 85, 90 (X in the L2, 6304 x 768 x 768: 11.5, 14.9). In the forward a tie
+  // goes to the added form: ViT-B, 128 images, K = 768 4.06 -> 4.02 ms. Read ahead
+  // too on a nearly idle chip, where the read hides behind the main loop and a
+  // reduce-add completes later.
   const int rows = pair ? 2 * BM : BM;
   const long tiles = static_cast<long>((Mt + rows - 1) / rows) * ((N + a.bn - 1) / a.bn);
-  const bool memory_bound = K <= 1024 && 4.0 * Mt * N > 64e6;
+  const bool memory_bound = K <= 700 && 4.0 * Mt * N > 64e6;
   if (epi == EPI_BIAS_ADD_F32 && (memory_bound || 4 * tiles <= (pair ? sms / 2 : sms))) epi = EPI_BIAS_RESID_F32;
   p->epi = epi;
   if (tma_out) {
