@@ -36,10 +36,10 @@
 //    registers. GELU, bias and residual use packed fp32 pairs.
 //    * the fp32 residual stream (out-proj, FC2) leaves by TMA reduce-add, from
 //      eight warps: X is not read into the SM. FC2 (K = 3072, 50432 rows) 154 ->
-//      142 us, K = 1536 92 -> 86. Where memory sets the pace, and in a plan of
-//      few tiles, the old rows are read into the staging pieces ahead instead
-//      (out-proj 72 -> 68), as the 16-bit residual + ReLU of the CNN block
-//      outputs are.
+//      142 us, K = 1536 92 -> 85. Where memory sets the pace (K <= 700), and in a
+//      plan of few tiles, the old rows are read into the staging pieces ahead
+//      instead (K = 192 64.5 -> 54.7), as the 16-bit residual + ReLU of the CNN
+//      block outputs are.
 //    * a split-K plan (k-block range tile / (mt * nt)) stores fp32 partial sums
 //      the same way; the transposing epilogue took its CTAs 2.5 us of a 4.9 us
 //      one-image launch.
