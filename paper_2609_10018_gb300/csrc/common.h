@@ -139,6 +139,7 @@ struct HaloArgs {
   int Ho, Wo, bw, bh, nbx, nby; // output size, pixel block of a CTA (bw x bh), blocks across and down an image
   int wp;                       // halo width: pixels between two halo rows in shared memory
   int taps_x, taps_y, cgroups, pad;
+  int tap_stride;               // filter values between two taps: 64 * cgroups, or 16 (at most 16 channels, 3 x 3)
   int a_tx, a_stage, a_stages;  // bytes of a halo load and of its ring stage, stages
   int b_stages, b_resident;     // filter ring depth, or the whole filter kept in shared memory
   const float* bias;

@@ -30,9 +30,9 @@
 // accumulators instead of two (72).
 // Back-to-back calls, box per tap -> here: 128 images of 56 x 56 x 64 -> 64
 // channels 67.5 -> 26.5 us (35.9 with the taps in a loop), 28 x 28 x 128 -> 128
-// 35.3 -> 20.5 us (1.45 PFLOP/s), 28 x 28 x 96 -> 96 35.5 -> 16.8, 14 x 14 x 192 ->
+// 35.3 -> 20.5 us (1.45 PFLOP/s), 28 x 28 x 96 -> 96 35.5 -> 16.8, 56 x 56 x 16 -> 16 47.9 -> 20.9, 14 x 14 x 192 ->
 // 192 20.5 -> 17.0, 16 images of 56 x 56 x 64 12.3 -> 7.5 us. 7 x 7 images (49 of
-// 128 rows) and at most 16 channels stay with the box per tap. So do strides: the
+// 128 rows) stay with the box per tap. So do strides: the
 // four parity tiles of a 3 x 3 of stride 2 hold one to four taps each (100 images
 // of 28 x 28 x 192 at stride 2: 23.7 us on such tiles, 19.0 with a box per tap).
 #include <algorithm>
@@ -103,13 +103,16 @@ struct TileWalk {
   }
 };
 
-// TX x TY taps known at compile time (3 x 3, and the stem's 1 x 4), or 0.
-template <bool RELU, int TX, int TY>
+// TX x TY taps known at compile time (3 x 3, and the stem's 1 x 4), or 0. KS: K =
+// 16 steps of a tap; 1 for at most 16 channels, whose filter box runs into the
+// next taps past them (never read).
+template <bool RELU, int TX, int TY, int KS = 4>
 __global__ void __launch_bounds__(THREADS, 1)
     conv_halo_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                      const HaloArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  constexpr int KSTRIDE = KS == 1 ? 16 : 64;  // filter values between two k-blocks
   const int taps = a.taps_x * a.taps_y, nk = taps * a.cgroups;
   const int half = a.bn / 2;            // filter rows of one CTA's k-block
   const int b_bytes = half * 128;
@@ -169,7 +172,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (a.b_resident && warp == 0 && t0 < tiles && elect_one()) {
     if (leader) mbar_expect_tx(&b_full[0], 2u * nk * b_bytes);
     const uint32_t bar = cluster_map(smem_addr(&b_full[0]), 0);
-    for (int k = 0; k < nk; ++k) tma_load_2d_pair(sB + k * b_bytes, &tmW, bar, k * 64, rank * half);
+    for (int k = 0; k < nk; ++k) tma_load_2d_pair(sB + k * b_bytes, &tmW, bar, k * KSTRIDE, rank * half);
   }
   if (warp != 10 || a.b_resident) {
     pdl_wait();
@@ -228,7 +231,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             if (leader) mbar_expect_tx(&b_full[s], 2u * b_bytes);
             tma_load_2d_pair(sB + s * b_bytes, &tmW, cluster_map(smem_addr(&b_full[s]), 0),
-                             (tap * a.cgroups + g) * 64, row);
+                             (tap * a.cgroups + g) * KSTRIDE, row);
             ++issued;
             if (++s == a.b_stages) {
               s = 0;
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t a_lo = a_base + as * (a.a_stage >> 4), wp8 = 8u * a.wp;
           auto tap_mma = [&](uint32_t lo, uint32_t b_lo, uint32_t accumulate) {
 #pragma unroll
-            for (uint32_t k = 0; k < 4; ++k)
+            for (uint32_t k = 0; k < KS; ++k)
               tc_mma_pair_warp_lo(d, lo + 2 * k, b_lo + 2 * k, hi, idesc, k > 0 ? 1u : accumulate);
           };
           auto streamed_tap = [&](uint32_t lo, uint32_t accumulate) -> bool {
@@ -448,7 +451,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 }
 
 using HaloKernel = void (*)(CUtensorMap, CUtensorMap, HaloArgs);
-HaloKernel halo_kernel(bool relu, int taps_x, int taps_y) {
+HaloKernel halo_kernel(bool relu, int taps_x, int taps_y, bool narrow) {
+  if (narrow) return relu ? conv_halo_kernel<true, 3, 3, 1> : conv_halo_kernel<false, 3, 3, 1>;
   if (taps_x == 3 && taps_y == 3) return relu ? conv_halo_kernel<true, 3, 3> : conv_halo_kernel<false, 3, 3>;
   if (taps_x == 1 && taps_y == 4) return relu ? conv_halo_kernel<true, 1, 4> : conv_halo_kernel<false, 1, 4>;
   return relu ? conv_halo_kernel<true, 0, 0> : conv_halo_kernel<false, 0, 0>;
@@ -462,10 +466,11 @@ cudaError_t halo_init_attributes() {
   const int bytes = static_cast<int>(SMEM_BYTES);
   cudaError_t e = cudaSuccess;
   for (int relu = 0; relu < 2; ++relu)
-    for (int t = 0; t < 3; ++t)
+    for (int t = 0; t < 4; ++t) {
+      const HaloKernel k = halo_kernel(relu != 0, t == 2 ? 1 : t == 0 ? 0 : 3, t == 2 ? 4 : t == 0 ? 0 : 3, t == 3);
       if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(halo_kernel(relu != 0, t == 2 ? 1 : 3 * t, t == 2 ? 4 : 3 * t)),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    }
   return e;
 }
 
@@ -548,7 +553,7 @@ bool halo_maps(GemmPlan* p, const void* x, const uint64_t xd[4], const uint64_t 
   const HaloArgs& a = p->halo;
   const uint32_t box[4] = {64u, static_cast<uint32_t>(a.wp), static_cast<uint32_t>(a.bh + a.taps_y - 1), 1u};
   const uint32_t es[4] = {1u, 1u, 1u, 1u};
-  const uint64_t K = static_cast<uint64_t>(a.taps_x) * a.taps_y * a.cgroups * 64;
+  const uint64_t K = static_cast<uint64_t>(a.taps_x) * a.taps_y * a.tap_stride;
   return encode_tmap_4d(&p->tmA, x, xd, xs, box, es, false) &&
          encode_tmap_2d(&p->tmB, Wt, K, a.N, K * 2, 64, a.bn / 2);
 }
@@ -572,7 +577,7 @@ cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, halo_kernel(p.epi == EPI_BIAS_RELU_F16, a.taps_x, a.taps_y), p.tmA, p.tmB, a);
+  return cudaLaunchKernelEx(&cfg, halo_kernel(p.epi == EPI_BIAS_RELU_F16, a.taps_x, a.taps_y, a.tap_stride < 64), p.tmA, p.tmB, a);
 }
 
 }  // namespace elasto

@@ -1225,12 +1225,16 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
   a.b_resident = (N <= a.bn && 4 * A_STAGE + b_all + CBUF <= POOL) ? 1 : 0;
   if (!a.b_resident && !k16) choose_tile(prob, 64, true, &a.bn, &pair);
   a.pair = pair ? 1 : 0;
-  // halo tiles where they are estimated faster than a box per tap
+  // halo tiles where they are estimated faster than a box per tap (a 16-channel
+  // box takes as long as a 64-channel one: counted as a k-block per tap); their
+  // offsets within an image are 32-bit, in 16-byte units
   double halo = 0.0;
-  // (its offsets within an image are 32-bit, in 16-byte units)
-  if (!k16 && stride == 1 && static_cast<int64_t>(Ho) * Wo * ldo < (int64_t(1) << 34) &&
+  Problem boxes = prob;
+  boxes.K = nk * BK;
+  if ((!k16 || (taps_x == 3 && taps == 9)) && stride == 1 && static_cast<int64_t>(Ho) * Wo * ldo < (int64_t(1) << 34) &&
       halo_layout(&p->halo, B_cap, Ho, Wo, taps_x, taps / taps_x, cg, pad, N, prob.sms, &halo) &&
-      halo < tile_cost(prob, a.bn, pair)) {
+      halo < tile_cost(boxes, a.bn, pair)) {
+    p->halo.tap_stride = cg * bke;
     p->halo.bias = bias;
     p->halo.out = out;
     p->halo.ldo = ldo;

@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
     (9, 14, 14, 256, 520, 3, 1, True),     # filter streamed, three filter tiles, the last 8 channels wide
     (2, 17, 140, 24, 16, 5, 2, True),      # 5 x 5, image wider than a block
     (4, 8, 8, 256, 64, 2, 0, False),       # even kernel
+    (128, 56, 56, 16, 16, 3, 1, True),     # 16-wide filter taps: one K step a tap
+    (128, 31, 29, 8, 24, 3, 1, False),     # half a K step
 ])
 def test_halo_convolution_matches_fp64(B, H, W, C, N, k, pad, relu):
     import torch
@@ -25,7 +27,7 @@ def test_halo_convolution_matches_fp64(B, H, W, C, N, k, pad, relu):
     x = rng.standard_normal((B, H, W, C)).astype(np.float16)
     w = (rng.standard_normal((N, C, k, k)) * np.sqrt(2.0 / (C * k * k))).astype(np.float16)
     bias = (rng.standard_normal(N) * 0.1).astype(np.float32)
-    packed = np.zeros((N, k, k, (C + 63) // 64 * 64), np.float16)
+    packed = np.zeros((N, k, k, 16 if C <= 16 else (C + 63) // 64 * 64), np.float16)
     packed[..., :C] = w.transpose(0, 2, 3, 1)
     ref = orr.conv2d(x.astype(np.float64), w.astype(np.float64), 1, pad) + bias
     if relu:
