@@ -120,7 +120,10 @@ __device__ __forceinline__ float softmax_row(uint32_t tm, int n) {
   }
   const float neg = -fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])) * kScale;
   const float2 scale2 = make_float2(kScale, kScale), neg2 = make_float2(neg, neg);
-  float2 s[4] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+  // four partial sums, each of the key pairs 4 i + its number: neighbours are
+  // added to one another first, which keeps numerators too small to change the
+  // partial sum one by one
+  float2 s[2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
   if constexpr (NF > 0) load64(tm, v[0]);
 #pragma unroll
   for (int i = 0; i < NF; ++i) {
@@ -130,12 +133,17 @@ __device__ __forceinline__ float softmax_row(uint32_t tm, int n) {
       if (i + 1 < NF) tmem_ld_32x32b_x32(tm + 64 * (i + 1) + 32 * h, v[(i + 1) & 1][h]);
       uint32_t pk[16];
 #pragma unroll
-      for (int j = 0; j < 32; j += 2) {
-        const float2 x = fma2(make_float2(__uint_as_float(v[i & 1][h][j]), __uint_as_float(v[i & 1][h][j + 1])), scale2,
-                              neg2);
-        const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
-        s[(j >> 1) & 3] = add2(s[(j >> 1) & 3], p);
-        pk[j >> 1] = pack_bf16x2(p.x, p.y);
+      for (int j = 0; j < 32; j += 4) {
+        float2 p[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int e = j + 2 * k;
+          const float2 x = fma2(make_float2(__uint_as_float(v[i & 1][h][e]), __uint_as_float(v[i & 1][h][e + 1])),
+                                scale2, neg2);
+          p[k] = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+          pk[e >> 1] = pack_bf16x2(p[k].x, p[k].y);
+        }
+        s[(j >> 2) & 1] = add2(s[(j >> 2) & 1], add2(make_float2(p[0].x, p[1].x), make_float2(p[0].y, p[1].y)));
       }
       tmem_st_16(tm + 32 * i + 16 * h, pk);
     }
@@ -145,16 +153,20 @@ __device__ __forceinline__ float softmax_row(uint32_t tm, int n) {
     tmem_ld_16(tm + c, w);
     tmem_ld_wait();
 #pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-      const float2 x = fma2(make_float2(__uint_as_float(w[j]), __uint_as_float(w[j + 1])), scale2, neg2);
-      const float2 p = make_float2(c + j < n ? ex2_approx(x.x) : 0.0f, c + j + 1 < n ? ex2_approx(x.y) : 0.0f);
-      s[(j >> 1) & 3] = add2(s[(j >> 1) & 3], p);
-      pk[j >> 1] = pack_bf16x2(p.x, p.y);
+    for (int j = 0; j < 16; j += 4) {
+      float2 p[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int e = j + 2 * k;
+        const float2 x = fma2(make_float2(__uint_as_float(w[e]), __uint_as_float(w[e + 1])), scale2, neg2);
+        p[k] = make_float2(c + e < n ? ex2_approx(x.x) : 0.0f, c + e + 1 < n ? ex2_approx(x.y) : 0.0f);
+        pk[e >> 1] = pack_bf16x2(p[k].x, p[k].y);
+      }
+      s[(j >> 2) & 1] = add2(s[(j >> 2) & 1], add2(make_float2(p[0].x, p[1].x), make_float2(p[0].y, p[1].y)));
     }
     tmem_st_8(tm + (c >> 1), pk);
   }
-  const float2 t = add2(add2(s[0], s[1]), add2(s[2], s[3]));
-  return t.x + t.y;
+  return (s[0].x + s[0].y) + (s[1].x + s[1].y);
 }
 
 __global__ void __launch_bounds__(THREADS, 1)

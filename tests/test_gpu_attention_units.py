@@ -35,3 +35,23 @@ def test_attention_units_match_fp64(B, n, h):
         ref = np.concatenate([ov.attention(q[:, 0, j], q[:, 1, j], q[:, 2, j], 64) for j in range(h)], axis=-1)
         # P and O are rounded to bf16 (2^-9 each, relative)
         assert np.max(np.abs(got[b] - ref)) <= 1e-2 * np.max(np.abs(ref)), (b, float(np.max(np.abs(got[b] - ref))))
+
+
+@pytest.mark.parametrize("n", [256, 255])
+def test_row_sum_keeps_small_numerators(n):
+    """Four keys with numerator 1, the rest 0.98 * 2^-24 each: too small to change
+    a partial sum near 1 alone, not in pairs. The values put every output at a
+    bf16 rounding tie plus 24 * 2^-23 relative, between the exact denominator
+    (30.9 * 2^-23 over 4) and the 15.7 * 2^-23 that is left where every second
+    numerator is lost."""
+    import torch
+    x = np.zeros((1, n, 3, 1, 64), np.float32)
+    x[..., 0, 0, :2] = 1.0
+    x[..., 1, 0, :2] = (-133.0, -0.25)  # exp(-133.25 / 8) = 0.98 * 2^-24
+    x[:, 0:8:2, 1] = 0.0
+    for key, value in ((0, 1.0), (2, 2.0 ** -8), (4, 24 * 2.0 ** -23)):
+        x[:, key, 2] = value
+    dq, out = dev(synth.f32_to_bf16_bits(x)), empty_dev((1, n, 64), torch.uint16)
+    binding.elasto_op_attention(stream_handle(), dq.data_ptr(), out.data_ptr(), 1, n, 1)
+    torch.cuda.synchronize()
+    assert np.all(bf16_to_f64(out) == 0.25)
