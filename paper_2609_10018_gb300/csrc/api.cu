@@ -795,6 +795,7 @@ elasto_status vit_create(const elasto_model_desc* d, const elasto_weights* wts, 
       set.rows[i] = h->plan_rows[i];
       const elasto_status r = make(set.plan[i], set.rows[i]);
       if (r != ELASTO_OK) return r;
+      set.plan[i].weights_constant();
     }
     return ELASTO_OK;
   };

@@ -686,6 +686,7 @@ elasto_status cnn_create(const elasto_model_desc* d, const elasto_weights* wts, 
   elasto_status st = gemm_plan_conv_rows(&m->stem, m->s2d, Bm, m->h1 + 3, m->w1 + 3, kS2dC, 4, 4, m->stem_w, kStemC,
                                          m->stem_b, m->xb, kStemC, EPI_BIAS_RELU_F16, m->status);
   if (st != ELASTO_OK) return st;
+  m->stem.weights_constant();
   m->down.assign(nblk, GemmPlan{});
   const int64_t stem_macs = int64_t(m->h1) * m->w1 * kStemC * kStemK + int64_t(2048) * C;
   for (int i = 0; i < nblk; ++i) {
@@ -700,6 +701,7 @@ elasto_status cnn_create(const elasto_model_desc* d, const elasto_weights* wts, 
         st = gemm_plan_conv(&m->down[i], xin, Bm, b.hin, b.win, b.cin, 1, b.stride, 0, m->down_w[i], 4 * b.w,
                             m->down_b[i], m->sc, 4 * b.w, EPI_BIAS_F16, m->status);
       if (st != ELASTO_OK) return st;
+      m->down[i].weights_constant();
     }
   }
   for (int mo = 0; mo < n_modes; ++mo) {
@@ -726,6 +728,7 @@ elasto_status cnn_create(const elasto_model_desc* d, const elasto_weights* wts, 
       if (st != ELASTO_OK) return st;
       st = gemm_set_residual_source(&bp.conv3, b.proj ? m->sc : xin, mo_cap);
       if (st != ELASTO_OK) return st;
+      for (GemmPlan* g : {&bp.conv1, &bp.conv2, &bp.conv3}) g->weights_constant();
       cm.macs += int64_t(b.hin) * b.win * bp.a * b.cin + int64_t(b.ho) * b.wo * bp.b * 9 * bp.a +
                  int64_t(b.ho) * b.wo * 4 * b.w * bp.b + (b.proj ? int64_t(b.ho) * b.wo * 4 * b.w * b.cin : 0);
       cm.launches += 3 + (b.proj ? 1 : 0);

@@ -111,6 +111,7 @@ struct GemmArgs {
   int cbufs;              // output staging pieces (4 KB) of each epilogue warp, for the TMA-store epilogues
   int b_planes;           // 2: W held as bf16 hi + lo planes (fp32-stored models), both multiplied
   int pair;               // 1: clusters of two CTAs sharing 256-row tiles (tcgen05 cta_group::2)
+  int w_const;            // 1: no earlier kernel writes W, so it is read before the wait for that kernel
   int f16;                // 1: A, W, the residual and 16-bit outputs are f16 (the *_F16 epilogues), else bf16
   // Implicit-GEMM convolution (conv != 0): A is never materialised. An M
   // tile is a block of bw x bh output pixels of nb images; k-block kb = (tap,
@@ -142,6 +143,7 @@ struct HaloArgs {
   int tap_stride;               // filter values between two taps: 64 * cgroups, or 16 (at most 16 channels, 3 x 3)
   int a_tx, a_stage, a_stages;  // bytes of a halo load and of its ring stage, stages
   int b_stages, b_resident;     // filter ring depth, or the whole filter kept in shared memory
+  int w_const;                  // as in GemmArgs
   const float* bias;
   void* out;  // f16 [batch, Ho, Wo, ldo]
   int ldo;
@@ -168,6 +170,9 @@ struct GemmPlan {
   const float* ln_b = nullptr;
   bf16* ln_y = nullptr;
   int ln_d = 0;
+  // For a model's own packed weights: a launch loads W while the kernel before
+  // it is still running. A caller's W may be that kernel's output.
+  void weights_constant() { args.w_const = halo.w_const = 1; }
 };
 
 // Build maps/arguments for out = epi(A[M_cap, K] W[N, K]^T). A and W must stay

@@ -167,14 +167,16 @@ __global__ void __launch_bounds__(THREADS, 1)
   cluster_sync_all();  // both CTAs' barriers initialised before any remote arrive
   tc_fence_after();
   const uint32_t tmem = warp_uniform(static_cast<int>(*tmem_slot));
-  // The filter is not written by an earlier kernel of a stream that triggers
-  // early: its producers start before the wait for that kernel.
+  // A model's filter is not written by an earlier kernel of the stream
+  // (w_const): its producers start before the wait for that kernel.
   if (a.b_resident && warp == 0 && t0 < tiles && elect_one()) {
+    if (!a.w_const) pdl_wait();
     if (leader) mbar_expect_tx(&b_full[0], 2u * nk * b_bytes);
     const uint32_t bar = cluster_map(smem_addr(&b_full[0]), 0);
     for (int k = 0; k < nk; ++k) tma_load_2d_pair(sB + k * b_bytes, &tmW, bar, k * KSTRIDE, rank * half);
   }
-  if (warp != 10 || a.b_resident) {
+  const bool early = warp == 10 && !a.b_resident && a.w_const;
+  if (!early) {
     pdl_wait();
     pdl_trigger();
   }
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       for (long i = issued > a.b_stages ? issued - a.b_stages : 0; leader && i < issued; ++i)
         mbar_wait(&b_full[i % a.b_stages], static_cast<uint32_t>((i / a.b_stages) & 1));
     }
-    if (!a.b_resident) {
+    if (early) {
       pdl_wait();
       pdl_trigger();
     }

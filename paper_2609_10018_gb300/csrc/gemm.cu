@@ -280,8 +280,8 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
   const uint32_t tmem_base = warp_uniform(static_cast<int>(*tmem_slot));
   // Everything above overlapped the previous kernel's tail. Every thread
   // waits for that kernel (pdl_wait) before its first access to data it may
-  // write; the weights are not such data, so the producer thread starts
-  // loading them first and waits after that.
+  // write; a model's weights are not such data (w_const), so the producer
+  // thread starts loading them first and waits after that.
   if (warp != 0 || nk == 0) {
     pdl_wait();
     pdl_trigger();
@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
       const uint32_t a_bytes = args.conv ? args.cv_a_bytes : A_STAGE;
       const uint32_t bytes = PAIR ? 2 * (a_bytes + (bn / 2) * BK * 2) : a_bytes + (bres ? 0 : NB * bn * bke * 2);
       const bool b_loaded = bres && t_start < tiles && pid == 0;
+      if (!args.w_const) pdl_wait();
       if (b_loaded) {  // all of W, once: nk k-blocks of the single N tile
         mbar_expect_tx(bfull, static_cast<uint32_t>(nk) * bn * bke * 2);
         for (int kb = 0; kb < nk; ++kb) tma_load_2d(sB + kb * BSTG, &tmB, bfull, kb * bke, 0);

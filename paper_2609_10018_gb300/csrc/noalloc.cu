@@ -162,6 +162,7 @@ elasto_status build_plans(elasto_s* h, int mode, int batch, char* base, const Sc
   if (st != ELASTO_OK) return st;
   st = gemm_set_residual_source(&P->patch, em.pruned ? em.addend : h->tok_addend, h->addend_rows, n);
   if (st != ELASTO_OK) return st;
+  P->patch.weights_constant();
   P->layers.assign(vm.layers.size(), NoallocLayerPlans{});
   for (size_t l = 0; l < vm.layers.size(); ++l) {
     const VitLayerPack& lp = vm.layers[l];
@@ -181,6 +182,7 @@ elasto_status build_plans(elasto_s* h, int mode, int batch, char* base, const Sc
     if ((st = gemm_plan(&q.fc2, H, M, lp.fc2_w, D, lp.f_pad, em.fc2_b[l], X, D, EPI_BIAS_RESID_F32, h->status,
                         lp.fc2_w_lo, M, lp.ld_fc2)) != ELASTO_OK)
       return st;
+    for (GemmPlan* g : {&q.qkv, &q.proj, &q.fc1, &q.fc2}) g->weights_constant();
   }
   return ELASTO_OK;
 }
