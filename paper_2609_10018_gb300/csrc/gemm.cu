@@ -1240,7 +1240,8 @@ elasto_status plan_conv_common(GemmPlan* p, const char* who, const void* x, cons
     p->halo.out = out;
     p->halo.ldo = ldo;
     p->halo.status = status;
-    if (!halo_maps(p, x, xd, xs, Wt)) {
+    // (the output has no map that would refuse its address: it is stored by 16-byte pieces)
+    if (reinterpret_cast<uintptr_t>(out) % 16 != 0 || !halo_maps(p, x, xd, xs, Wt)) {
       set_error(std::string(who) + ": cuTensorMapEncodeTiled failed (alignment or size)");
       return ELASTO_ERR_UNSUPPORTED;
     }

@@ -44,3 +44,16 @@ def test_halo_convolution_matches_fp64(B, H, W, C, N, k, pad, relu):
     assert np.all(np.isfinite(got))
     # one f16 rounding (2^-11 relative, doubled) and fp32 accumulation
     assert np.all(np.abs(got - ref) <= 2.0 ** -10 * np.abs(ref) + 1e-4 * np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("stride", [1, 2])  # halo tiles, and a box per tap
+@pytest.mark.parametrize("which", ["x", "w", "out"])
+def test_misaligned_pointers_are_refused(stride, which):
+    """Every pointer that is not 16-byte aligned is refused before a launch."""
+    import torch
+    buf = {k: torch.zeros(1 << 20, dtype=torch.float16, device="cuda") for k in ("x", "w", "out")}
+    ptr = {k: v.data_ptr() + (8 if k == which else 0) for k, v in buf.items()}
+    with pytest.raises(binding.ElastoError) as e:
+        binding.elasto_op_conv2d(stream_handle(), ptr["x"], 2, 28, 28, 64, ptr["w"], 64, 3, stride, 1, None, True,
+                                 ptr["out"])
+    assert e.value.status == binding.ERR_UNSUPPORTED
