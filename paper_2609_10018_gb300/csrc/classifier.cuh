@@ -89,7 +89,8 @@ __device__ __forceinline__ void prepare_rows(const float* __restrict__ x, size_t
   }
 }
 
-// grid (ceil(B / 8), ceil(C / 8)), 256 threads, 8 * d floats of shared memory.
+// grid (ceil(C / 8), ceil(B / 8)): classes along x, which alone reaches past
+// 65535 blocks; 256 threads, 8 * d floats of shared memory.
 template <bool LN, int NV>
 __global__ void __launch_bounds__(256) small_kernel(const float* __restrict__ X, size_t row, int B, int d, int d_true,
                                                     const float* __restrict__ g, const float* __restrict__ bta,
@@ -98,8 +99,8 @@ __global__ void __launch_bounds__(256) small_kernel(const float* __restrict__ X,
   extern __shared__ float4 smem4[];
   float* sy = reinterpret_cast<float*>(smem4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b0 = blockIdx.x * SMALL_IMGS, nimg = min(SMALL_IMGS, B - b0);
-  const int c = blockIdx.y * WARPS + warp;
+  const int b0 = blockIdx.y * SMALL_IMGS, nimg = min(SMALL_IMGS, B - b0);
+  const int c = blockIdx.x * WARPS + warp;
   const float* wr = W + static_cast<size_t>(min(c, C - 1)) * d;
   float4 w[NV];
 #pragma unroll
@@ -265,7 +266,7 @@ cudaError_t launch(const float* X, size_t row, int B, int d, int d_true, const f
     return launch_pdl(tile_kernel<LN>, dim3(gx, LN && most < gy ? (most > 1 ? most : 1) : gy), dim3(256),
                       tile_smem(LN, d), s, X, row, B, d, d_true, g, b, W, bias, C, logits);
   }
-  return launch_pdl(small_kernel<LN, NV>, dim3((B + SMALL_IMGS - 1) / SMALL_IMGS, (C + WARPS - 1) / WARPS), dim3(256),
+  return launch_pdl(small_kernel<LN, NV>, dim3((C + WARPS - 1) / WARPS, (B + SMALL_IMGS - 1) / SMALL_IMGS), dim3(256),
                     SMALL_IMGS * d * sizeof(float), s, X, row, B, d, d_true, g, b, W, bias, C, logits);
 }
 

@@ -45,6 +45,7 @@ def test_resnet_odd_sizes(img, batch, classes, dtype):
     (16, 33, 192, 3),    # smallest batch of the tiled one, one class past a tile
     (65, 45, 320, 5),    # one image past two tiles, d not a multiple of a chunk
     (1, 1000, 1024, 16),  # widest row
+    (2, 600000, 64, 1),   # more groups of 8 classes than a grid has rows
 ])
 def test_vit_classifier_tiles(batch, classes, dim, heads):
     cfg = synth.vit_small_variant(synth.TINY, dim=dim, heads=heads, mlp=64, layers=1, classes=classes,
