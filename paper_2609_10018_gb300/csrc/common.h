@@ -30,6 +30,11 @@ elasto_status cuda_fail(cudaError_t e, const char* what);  // records "<what>: <
 int num_sms();  // of the current device
 
 // ---------------------------------------------------------------- launches
+// CTA pairs of `kernel` that the current device runs at once (at most one CTA
+// an SM; fewer than half the SMs where a group of SMs is odd). Every such
+// kernel takes an SM's whole shared memory, so one answer per device serves all.
+cudaError_t max_cta_pairs(const void* kernel, int threads, size_t smem, int* pairs);
+
 // Programmatic dependent launch. A kernel launched with launch_pdl may be
 // scheduled while the kernel before it on the stream is still finishing, so
 // its prologue (barrier set-up, TMEM allocation, descriptor prefetch) overlaps

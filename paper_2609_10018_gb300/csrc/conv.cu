@@ -564,7 +564,11 @@ cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s) {
   HaloArgs a = p.halo;
   a.batch = batch;
   const int nt = (a.N + a.bn - 1) / a.bn, blocks = batch * a.nby * a.nbx;
-  const int clusters = std::min((blocks + 1) / 2 * nt, num_sms() / 2);
+  const HaloKernel kernel = halo_kernel(p.epi == EPI_BIAS_RELU_F16, a.taps_x, a.taps_y, a.tap_stride < 64);
+  int pairs = 0;
+  const cudaError_t e = max_cta_pairs(reinterpret_cast<const void*>(kernel), THREADS, SMEM_BYTES, &pairs);
+  if (e != cudaSuccess) return e;
+  const int clusters = std::min((blocks + 1) / 2 * nt, pairs);
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -579,7 +583,7 @@ cudaError_t halo_launch(const GemmPlan& p, int batch, cudaStream_t s) {
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, halo_kernel(p.epi == EPI_BIAS_RELU_F16, a.taps_x, a.taps_y, a.tap_stride < 64), p.tmA, p.tmB, a);
+  return cudaLaunchKernelEx(&cfg, kernel, p.tmA, p.tmB, a);
 }
 
 }  // namespace elasto

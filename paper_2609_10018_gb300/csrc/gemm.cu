@@ -50,6 +50,7 @@
 //    output is stored by 4-D boxes of the tile's pixel block.
 //  Every mbarrier wait is bounded; a timeout records ELASTO_ERR_TIMEOUT.
 #include <algorithm>
+#include <atomic>
 
 #include "act.cuh"
 #include "common.h"
@@ -854,9 +855,12 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
   a.cv_batch = M;  // implicit convolutions: M counts images
   const int nt = (a.N + a.bn - 1) / a.bn;
   if constexpr (PAIR) {
-    static int max_clusters[64] = {0};  // (one CTA per SM by shared memory, whatever its threads)
-    int dev = 0;
-    cudaGetDevice(&dev);
+    const int threads = a.conv ? THREADS_CONV : epi_threads(EPI);
+    int pairs = 0;
+    const cudaError_t e = max_cta_pairs(reinterpret_cast<const void*>(gemm_tc_kernel<EPI, NB, true>), threads,
+                                        SMEM_BYTES, &pairs);
+    if (e != cudaSuccess) return e;
+    const int tiles = (a.conv ? (conv_mtiles(a) + 1) / 2 : (M + 2 * BM - 1) / (2 * BM)) * nt;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -865,21 +869,11 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_pdl
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.blockDim = dim3(a.conv ? THREADS_CONV : epi_threads(EPI));
+    cfg.gridDim = dim3(2 * std::min(tiles, pairs));
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;  // the occupancy query sees the cluster shape only
-    if (dev >= 0 && dev < 64 && max_clusters[dev] == 0) {
-      cfg.gridDim = dim3(2 * (num_sms() / 2));
-      int n = 0;
-      cudaError_t e = cudaOccupancyMaxActiveClusters(&n, gemm_tc_kernel<EPI, NB, true>, &cfg);
-      if (e != cudaSuccess || n <= 0) return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
-      max_clusters[dev] = n;
-    }
-    const int tiles = (a.conv ? (conv_mtiles(a) + 1) / 2 : (M + 2 * BM - 1) / (2 * BM)) * nt;
-    const int clusters = tiles < max_clusters[dev] ? tiles : max_clusters[dev];
-    cfg.gridDim = dim3(2 * clusters);
     cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI, NB, true>, p.tmA, p.tmB, p.tmB2, p.tmC, p.tmR, a);
   } else {
@@ -892,6 +886,32 @@ cudaError_t launch_epi(const GemmPlan& p, int M, cudaStream_t s) {
 }
 
 }  // namespace
+
+cudaError_t max_cta_pairs(const void* kernel, int threads, size_t smem, int* pairs) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  *pairs = known[dev].load(std::memory_order_relaxed);
+  if (*pairs > 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(2 * (num_sms() / 2));
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaOccupancyMaxActiveClusters(pairs, kernel, &cfg);
+  if (e != cudaSuccess) return e;
+  if (*pairs <= 0) return cudaErrorInvalidConfiguration;
+  known[dev].store(*pairs, std::memory_order_relaxed);
+  return cudaSuccess;
+}
 
 cudaError_t gemm_init_attributes() {
   const int bytes = static_cast<int>(SMEM_BYTES);
