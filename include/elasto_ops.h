@@ -67,6 +67,18 @@ elasto_status elasto_op_softmax(void* stream, const float* x, float* y, int rows
 elasto_status elasto_op_conv2d(void* stream, const void* x, int B, int H, int W, int C, const void* w, int N, int k,
                                int stride, int pad, const float* bias, int relu, void* out, int* status_device);
 
+/* The tiles that elasto_op_gemm / elasto_op_conv2d cut a call of this size into
+ * on the current device (16-byte aligned operands). Nothing is launched. */
+typedef struct {
+  int columns; /* output columns (channels) of a tile */
+  int pair;    /* 1: a pair of CTAs shares a tile of 256 rows; 0: a CTA has 128 rows of its own */
+  int halo;    /* 1: conv2d on halo tiles (always pairs); 0: a box of x per k-block */
+  int ahead;   /* pieces of 32 rows x 128 bytes of a residual that an epilogue warp reads ahead;
+                  0: no residual, or (RESID_F32) one that the stores add to */
+} elasto_tile;
+elasto_status elasto_op_gemm_tile(int M, int N, int K, int epilogue, elasto_tile* tile);
+elasto_status elasto_op_conv2d_tile(int B, int H, int W, int C, int N, int k, int stride, int pad, elasto_tile* tile);
+
 /* Multi-head attention over the kept heads (Eq. 3), all heads of width 64:
  * qkv bf16 [batch, n, 3, heads, 64] (q | k | v blocks, head-major, as the
  * QKV GEMM writes them) -> out bf16 [batch, n, heads * 64] (heads

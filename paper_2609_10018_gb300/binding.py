@@ -108,6 +108,8 @@ def lib() -> ctypes.CDLL:
                            c_void_p],
         "elasto_op_conv2d": [c_void_p, c_void_p, c_int, c_int, c_int, c_int, c_void_p, c_int, c_int, c_int, c_int,
                              c_void_p, c_int, c_void_p, c_void_p],
+        "elasto_op_gemm_tile": [c_int, c_int, c_int, c_int, c_void_p],
+        "elasto_op_conv2d_tile": [c_int, c_int, c_int, c_int, c_int, c_int, c_int, c_int, c_void_p],
         "elasto_op_layernorm": [c_void_p, c_void_p, c_void_p, c_void_p, c_void_p, c_int, c_int],
         "elasto_op_softmax": [c_void_p, c_void_p, c_void_p, c_int, c_int],
         "elasto_op_attention": [c_void_p, c_void_p, c_void_p, c_int, c_int, c_int, c_void_p],
@@ -378,6 +380,26 @@ def elasto_op_gemm(stream, A, W, bias, out, resid, M, N, K, epilogue, status=0) 
 def elasto_op_conv2d(stream, x, B, H, W, C, w, N, k, stride, pad, bias, relu, out, status=0) -> None:
     _check(lib().elasto_op_conv2d(stream, x, B, H, W, C, w, N, k, stride, pad, bias, int(relu), out, status),
            "elasto_op_conv2d")
+
+
+class Tile(ctypes.Structure):
+    """elasto_tile: how a GEMM or convolution call is cut up."""
+    _fields_ = [(f, c_int) for f in ("columns", "pair", "halo", "ahead")]
+
+    def fields(self) -> tuple:
+        return self.columns, self.pair, self.halo, self.ahead
+
+
+def elasto_op_gemm_tile(M, N, K, epilogue) -> Tile:
+    t = Tile()
+    _check(lib().elasto_op_gemm_tile(M, N, K, epilogue, ctypes.byref(t)), "elasto_op_gemm_tile")
+    return t
+
+
+def elasto_op_conv2d_tile(B, H, W, C, N, k, stride, pad) -> Tile:
+    t = Tile()
+    _check(lib().elasto_op_conv2d_tile(B, H, W, C, N, k, stride, pad, ctypes.byref(t)), "elasto_op_conv2d_tile")
+    return t
 
 
 def elasto_op_layernorm(stream, x, gamma, beta, y, rows, d) -> None:

@@ -99,6 +99,39 @@ elasto_status elasto_op_conv2d(void* stream, const void* x, int B, int H, int W,
   return ELASTO_OK;
 }
 
+elasto_status elasto_op_gemm_tile(int M, int N, int K, int epilogue, elasto_tile* tile) {
+  clear_error();
+  if (!tile || M <= 0 || N <= 0 || K < 0 || epilogue < 0 || epilogue > 8) {
+    set_error("elasto_op_gemm_tile: invalid arguments");
+    return ELASTO_ERR_INVALID_ARG;
+  }
+  elasto_status st = check_device();
+  if (st != ELASTO_OK) return st;
+  GemmPlan p;
+  bf16* const any = reinterpret_cast<bf16*>(uintptr_t(1) << 20);  // (encoded, never read)
+  st = gemm_plan(&p, any, M, any, N, K, nullptr, any, N, epilogue, nullptr);
+  if (st != ELASTO_OK) return st;
+  const bool ahead = p.epi == EPI_BIAS_RESID_F32 || p.epi == EPI_BIAS_RESID_RELU_BF16 || p.epi == EPI_BIAS_RESID_RELU_F16;
+  *tile = {p.args.bn, p.args.pair, 0, ahead ? p.args.cbufs : 0};
+  return ELASTO_OK;
+}
+
+elasto_status elasto_op_conv2d_tile(int B, int H, int W, int C, int N, int k, int stride, int pad, elasto_tile* tile) {
+  clear_error();
+  if (!tile || B <= 0 || H <= 0 || W <= 0 || C <= 0 || N <= 0 || k <= 0 || stride <= 0 || pad < 0) {
+    set_error("elasto_op_conv2d_tile: invalid arguments");
+    return ELASTO_ERR_INVALID_ARG;
+  }
+  elasto_status st = check_device();
+  if (st != ELASTO_OK) return st;
+  GemmPlan p;
+  void* const any = reinterpret_cast<void*>(uintptr_t(1) << 20);  // (encoded, never read)
+  st = gemm_plan_conv(&p, any, B, H, W, C, k, stride, pad, any, N, nullptr, any, N, EPI_BIAS_F16, nullptr);
+  if (st != ELASTO_OK) return st;
+  *tile = {p.use_halo ? p.halo.bn : p.args.bn, p.use_halo ? 1 : p.args.pair, p.use_halo ? 1 : 0, 0};
+  return ELASTO_OK;
+}
+
 elasto_status elasto_op_layernorm(void* stream, const float* x, const float* gamma, const float* beta, void* y,
                                   int rows, int d) {
   clear_error();

@@ -1,7 +1,8 @@
 """The GEMM's tile variants at their edges, against fp64: CTA pairs at short
 reductions with ragged last rows and columns, the residual added by the store
 or read ahead, CNN block outputs, and convolutions on pairs whose last pixel
-block is missing."""
+block is missing. Each test first asserts that its sizes get the tile it is
+meant for: (columns, pair, halo, pieces read ahead)."""
 import numpy as np
 import pytest
 
@@ -17,16 +18,18 @@ def _bf16(rng, shape, scale=1.0):
     return synth.f32_to_bf16_bits(rng.standard_normal(shape, dtype=np.float32) * np.float32(scale))
 
 
-@pytest.mark.parametrize("M,N,K,epi", [
-    (19457, 2312, 768, binding.EPI_BIAS_BF16),       # pairs: one row and eight columns past the tiles
-    (19713, 520, 264, binding.EPI_BIAS_GELU_BF16),   # pairs, K a remainder of a k-block
-    (19713, 520, 1160, binding.EPI_BIAS_RESID_F32),  # pairs, residual added by the store
-    (25089, 776, 520, binding.EPI_BIAS_RESID_F32),   # pairs, short reduction past the L2: residual read ahead
-    (257, 64, 64, binding.EPI_BIAS_RESID_F32),       # few tiles: residual read ahead
-    (12289, 40, 192, binding.EPI_BIAS_RESID_F32),    # narrow single tiles
+@pytest.mark.parametrize("M,N,K,epi,tile", [
+    (19457, 2312, 768, binding.EPI_BIAS_BF16, (256, 1, 0, 0)),       # pairs: one row, eight columns past the tiles
+    (19457, 2312, 776, binding.EPI_BIAS_GELU_BF16, (256, 1, 0, 0)),  # pairs, K a remainder of a k-block
+    (19713, 520, 264, binding.EPI_BIAS_GELU_BF16, (192, 0, 0, 0)),   # single CTAs, ragged in every direction
+    (19713, 520, 1160, binding.EPI_BIAS_RESID_F32, (192, 1, 0, 0)),  # pairs, residual added by the store
+    (25089, 776, 520, binding.EPI_BIAS_RESID_F32, (160, 1, 0, 1)),   # pairs, short reduction past the L2: read ahead
+    (257, 64, 64, binding.EPI_BIAS_RESID_F32, (32, 0, 0, 2)),        # few tiles: residual read ahead
+    (12289, 40, 192, binding.EPI_BIAS_RESID_F32, (64, 0, 0, 0)),     # narrow single tiles
 ])
-def test_tile_edges_match_fp64(M, N, K, epi):
+def test_tile_edges_match_fp64(M, N, K, epi, tile):
     import torch
+    assert binding.elasto_op_gemm_tile(M, N, K, epi).fields() == tile
     rng = np.random.default_rng(M + N + K)
     A, W = _bf16(rng, (M, K)), _bf16(rng, (N, K), 0.05)
     bias = rng.standard_normal(N).astype(np.float32)
@@ -55,13 +58,16 @@ def test_tile_edges_match_fp64(M, N, K, epi):
     assert np.all(np.abs(got[rows] - ref) <= tol), float(np.max(np.abs(got[rows] - ref)))
 
 
-@pytest.mark.parametrize("B,S,C,N,k,stride", [
-    (77, 14, 136, 256, 3, 2),    # whole images per block (2 of 7 x 7): 39 blocks, the last pair has one
-    (51, 29, 200, 264, 3, 1),    # ragged pixel blocks and channels
-    (41, 28, 256, 512, 1, 2),    # strided projection
+@pytest.mark.parametrize("B,S,C,N,k,stride,tile", [
+    (109, 7, 520, 512, 3, 1, (256, 1, 0, 0)),   # pairs; two images per block: 55 blocks, the last pair has one
+    (99, 29, 200, 264, 3, 2, (192, 1, 0, 0)),   # pairs, strided; ragged pixel blocks and channels
+    (77, 14, 136, 256, 3, 2, (128, 0, 0, 0)),   # single CTAs, strided, two images per block
+    (41, 28, 256, 512, 1, 2, (192, 0, 0, 0)),   # single CTAs, strided projection
+    (51, 29, 200, 264, 3, 1, (144, 1, 1, 0)),   # halo tiles, ragged pixel blocks and channels
 ])
-def test_conv_pairs_match_fp64(B, S, C, N, k, stride):
+def test_conv_tiles_match_fp64(B, S, C, N, k, stride, tile):
     import torch
+    assert binding.elasto_op_conv2d_tile(B, S, S, C, N, k, stride, k // 2).fields() == tile
     rng = np.random.default_rng(B + S + C)
     x = rng.standard_normal((B, S, S, C)).astype(np.float16)
     w = (rng.standard_normal((N, C, k, k)) * np.sqrt(2.0 / (C * k * k))).astype(np.float16)
@@ -85,14 +91,18 @@ def test_conv_pairs_match_fp64(B, S, C, N, k, stride):
     assert np.all(np.abs(got[pick] - ref) <= 2.0 ** -10 * np.abs(ref) + 1e-4 * np.max(np.abs(ref)))
 
 
-@pytest.mark.parametrize("M,N,K", [
-    (100353, 264, 64),   # one k-block a tile: the residual read three pieces ahead
-    (25089, 1032, 200),  # past the L2, 128 columns
-    (6273, 2056, 520),   # 192 columns, one piece ahead
-    (129, 72, 64),       # one wave
+@pytest.mark.parametrize("M,N,K,tile", [
+    (100353, 248, 64, (128, 0, 0, 3)),    # one k-block a tile: the residual read three pieces ahead
+    (100353, 264, 64, (64, 0, 0, 3)),     # the same, narrow tiles
+    (25089, 1024, 200, (128, 0, 0, 2)),   # past the L2, 128 columns
+    (25089, 1032, 200, (192, 0, 0, 2)),   # 192 columns
+    (3137, 2056, 520, (192, 0, 0, 1)),    # 192 columns, one piece ahead
+    (6273, 2056, 520, (256, 0, 0, 1)),    # 256 columns
+    (129, 72, 64, (64, 0, 0, 3)),         # one wave
 ])
-def test_block_output_tiles_match_fp64(M, N, K):
+def test_block_output_tiles_match_fp64(M, N, K, tile):
     import torch
+    assert binding.elasto_op_gemm_tile(M, N, K, binding.EPI_BIAS_RESID_RELU_F16).fields() == tile
     rng = np.random.default_rng(M + N + K)
     A = rng.standard_normal((M, K), dtype=np.float32).astype(np.float16)
     W = (rng.standard_normal((N, K)) * np.sqrt(2.0 / K)).astype(np.float16)

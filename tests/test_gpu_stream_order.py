@@ -8,8 +8,9 @@ from paper_2609_10018_gb300 import binding
 pytestmark = pytest.mark.gpu
 
 
+# (a filter of one tile of 64 columns is kept in shared memory, more tiles are streamed)
 @pytest.mark.parametrize("kind,C,N,stride", [
-    ("conv", 64, 64, 1),     # halo tiles, filter kept in shared memory
+    ("conv", 64, 64, 1),     # halo tiles, filter kept
     ("conv", 256, 256, 1),   # halo tiles, filter streamed
     ("conv", 64, 64, 2),     # box per tap, filter kept
     ("conv", 256, 256, 2),   # box per tap, filter streamed
@@ -32,6 +33,7 @@ def test_weights_from_the_call_before(kind, C, N, stride):
                                binding.EPI_BIAS_F16)
 
     if kind == "conv":
+        assert binding.elasto_op_conv2d_tile(2, 28, 28, C, N, 3, stride, 1).fields() == (64, stride == 1, stride == 1, 0)
         x = f16(2, 28, 28, C)
         out = torch.empty((2, 28 // stride, 28 // stride, N), dtype=torch.float16, device="cuda")
 
