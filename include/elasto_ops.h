@@ -58,12 +58,14 @@ elasto_status elasto_op_softmax(void* stream, const float* x, float* y, int rows
  * stride + 1 (likewise Wo), act = ReLU if relu != 0 else identity.
  *   x f16 [B, H, W, C] NHWC, C % 8 == 0;
  *   w f16 [N, k, k, Cp] with Cp = 16 if C <= 16, else C rounded up to 64;
- *     channels >= C zero (the packed layout the ResNet path uses: one
- *     64-channel group per k-block of the tensor-core GEMM, or for at most 16
- *     channels one tap per 16-wide k-block in the 32-byte swizzle);
+ *     channels >= C zero (the packed layout the ResNet path uses: a k-block
+ *     of the tensor-core GEMM is one 64-channel group of a tap, or for at most
+ *     16 channels one tap);
  *   bias fp32 [N] or NULL. N % 2 == 0, stride 1 or 2.
- * No im2col buffer: each k-block is one 4-D TMA tile of x (padding read as
- * zeros, the stride by TMA traversal strides). */
+ * No im2col buffer: x is read by 4-D TMA tiles (padding read as zeros). At
+ * stride 1, N % 8 == 0 and where it is estimated faster, one tile per block of
+ * output pixels and channel group holds the pixels of all taps (its halo); else
+ * there is one per k-block, the stride by TMA traversal strides. */
 elasto_status elasto_op_conv2d(void* stream, const void* x, int B, int H, int W, int C, const void* w, int N, int k,
                                int stride, int pad, const float* bias, int relu, void* out, int* status_device);
 

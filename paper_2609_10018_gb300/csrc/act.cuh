@@ -29,7 +29,7 @@ __device__ __forceinline__ float gelu(float x) {
 }
 
 // Two values with packed fp32 instructions, bit-identical to two gelu calls:
-// 7 packed, 2 min and 4 MUFU instructions instead of 2 x 9.
+// 6 packed, 2 min and 4 MUFU instructions instead of 2 x 9.
 __device__ __forceinline__ float2 gelu2(float2 x) {
   float2 s = mul2(x, x);
   s = make_float2(fminf(s.x, 36.0f), fminf(s.y, 36.0f));

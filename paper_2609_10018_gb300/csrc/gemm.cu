@@ -589,8 +589,7 @@ __global__ void __launch_bounds__(epi_threads(EPI) + 32, 1)
           if (!ok) break;
           ++consumed;
         } else {
-          // the piece is free once the store that last read it (E chunks ago) has done so
-          if (elect_one()) E == 1 ? bulk_wait_read<0>() : bulk_wait_read<1>();
+          if (elect_one()) bulk_wait_read<0>();  // the one piece is free once its last store has read it
           if (args.conv)
             named_bar_sync(1 + g, 128);  // (one warp issues the group's stores)
           else
@@ -1008,8 +1007,8 @@ void choose_tile(const Problem& p, int step, bool pairs_allowed, int* bn, bool* 
 namespace {
 
 // Splits the pool between the operand ring and the epilogue's staging pieces.
-// cbufs counts pieces per epilogue warp: with a residual read through them (its
-// fetch depth) as many of two as leave 3 operand stages, 5 under an fp32 residual
+// cbufs counts pieces per epilogue warp: one, or with a residual read through them
+// (its fetch depth) as many of two as leave 3 operand stages, 5 under an fp32 residual
 // past 8 k-blocks and 4 under a 16-bit one past 4 (one piece, then two and fewer
 // stages: 50432 x 576 x 640 51.0 us, 53.6; 6272 x 2048 x 512 in 192 columns 15.7,
 // 16.7). A 16-bit residual's one-k-block tiles take three pieces and 2 stages
