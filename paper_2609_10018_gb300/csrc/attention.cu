@@ -34,7 +34,7 @@
 // What bounds it: each unit is a serial chain S -> softmax -> PV -> read-out and
 // TMEM holds two. ViT-B (256 images, 197 tokens, 12 heads), per unit: softmax
 // 2300 clocks (1660 of them the exponentials), PV 1000-1400, scaling and staging
-// O 900, S 300; 86.7 -> 61.9 us a call, the memory's share being 46. Before, the
+// O 900, S 300; 86.4 -> 61.8 us a call, the memory's share being 46. Before, the
 // softmax took 3700 (packed arithmetic and pipelined reads since) and storing
 // 16 bytes to each of 32 rows per instruction 1500-2000 (TMA boxes since). With
 // one query tile per item the second group had no work: 128 tokens 51.5 -> 34.3

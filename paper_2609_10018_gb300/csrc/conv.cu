@@ -28,11 +28,12 @@
 // additions (TileWalk; 128 images of 56 x 56 x 32 27.0 -> 24.3 us, the stem 81 ->
 // 70). Tried there without gain: a third group of epilogue warps (stem 73), four
 // accumulators instead of two (72).
-// Back-to-back calls, box per tap -> here: 128 images of 56 x 56 x 64 -> 64
-// channels 67.5 -> 26.5 us (35.9 with the taps in a loop), 28 x 28 x 128 -> 128
-// 35.3 -> 20.5 us (1.45 PFLOP/s), 28 x 28 x 96 -> 96 35.5 -> 16.8, 56 x 56 x 16 -> 16 47.9 -> 20.9, 14 x 14 x 192 ->
-// 192 20.5 -> 17.0, 16 images of 56 x 56 x 64 12.3 -> 7.5 us. 7 x 7 images (49 of
-// 128 rows) stay with the box per tap. So do strides: the
+// 400 calls back to back on one GPU, gemm.cu's box per tap on single CTAs -> here,
+// 128 images: 56 x 56 x 64 -> 64 channels 52.3 -> 25.9 us (35.9 with the taps in
+// a loop), 56 x 56 x 32 -> 32 48.9 -> 24.0, 56 x 56 x 16 -> 16 49.3 -> 19.7, 28 x
+// 28 x 128 -> 128 28.6 -> 20.1 (1.47 PFLOP/s), 28 x 28 x 96 -> 96 27.9 -> 16.4, 14
+// x 14 x 256 -> 256 28.0 -> 25.1, 14 x 14 x 192 -> 192 17.7 -> 16.9. 7 x 7 images
+// (49 of 128 rows) stay with the box per tap. So do strides: the
 // four parity tiles of a 3 x 3 of stride 2 hold one to four taps each (100 images
 // of 28 x 28 x 192 at stride 2: 23.7 us on such tiles, 19.0 with a box per tap).
 #include <algorithm>

@@ -22,9 +22,10 @@
 //    tile is shared memory: per k-block the MMAs read 48 KB and TMA writes
 //    48 KB, 0.38 us at 128 B a clock, more than the 0.27 us the MMAs take, and
 //    the epilogue's staging comes on top. A pair's CTA reads 32 KB and writes
-//    32 KB. ViT-B QKV at batch 256 (50432 x 2304 x 768): 124 us single, 108 us
-//    pairs; FC1 + GELU 172 -> 157 us; 50432 x 3072 x 768 without GELU 160 ->
-//    141 us (a library bf16 GEMM of that size: 140 us).
+//    32 KB. 400 calls back to back, the clock under the power cap: ViT-B QKV at
+//    batch 256 (50432 x 2304 x 768) 137 us single, 114 us pairs (a library bf16
+//    GEMM 101); FC1 + GELU 194 -> 170 us; 50432 x 3072 x 768 without GELU 188 ->
+//    165 us (library 156).
 //  - warps 2-13: epilogue, three warps per 32-lane quarter of TMEM (= 32 rows
 //    of the tile). A warp works alone: it takes every third 128-byte-wide
 //    chunk of its rows from TMEM to registers, writes it to its own 4 KB
@@ -49,6 +50,9 @@
 //    (one tap and channel group per k-block, padding read as zeros), and the
 //    output is stored by 4-D boxes of the tile's pixel block.
 //  Every mbarrier wait is bounded; a timeout records ELASTO_ERR_TIMEOUT.
+//  The two sides of a figure were taken in turn on one GPU. Figures of different
+//  steps are from different GPUs and run lengths, between which the power cap
+//  moves the clock, and the times of the large GEMMs by up to 12 %.
 #include <algorithm>
 #include <atomic>
 
@@ -971,7 +975,10 @@ double tile_cost(const Problem& p, int bn, bool pair) {
   const long tiles = static_cast<long>((p.M + rows - 1) / rows) * ((p.N + bn - 1) / bn);
   const long waves = (tiles + units - 1) / units;
   double load = stage_bytes(bn, pair, p.planes) / 126.0, mma = p.planes * (130.0 + 0.9 * bn);
-  if (p.conv) load = std::max(load, 280.0);  // 4-D boxes
+  // 4-D boxes. Narrow tiles advance at 230 to 260 ns a k-block (128 images of 56 x
+  // 56 x 64 in 64 columns 242); the margin decides for halo tiles up to 6 % too
+  // early on calls of 10 us (17 images of 31 x 31 x 32 -> 80 channels: 10.5, 9.8)
+  if (p.conv) load = std::max(load, 280.0);
   const double main_loop = ((p.K + BK - 1) / BK) * std::max(load, mma);
   const bool f32 = p.epi == EPI_BIAS_RESID_F32 || p.epi == EPI_BIAS_ADD_F32;
   double epilogue = 400.0 + bn * (f32 ? 8.0 : p.epi == EPI_BIAS_GELU_BF16 ? 9.0 : 6.0);
