@@ -35,7 +35,7 @@ GEMM_CASES = [
     # f16 operands (ResNet-50 path)
     (200, 48, 576, binding.EPI_BIAS_RELU_F16),        # 3x3 conv of 64 kept channels into 48
     (130, 16, 72, binding.EPI_BIAS_F16),              # N below one 64-column chunk
-    (1537, 256, 2048, binding.EPI_BIAS_RELU_F16),     # K >= 1536: CTA-pair kernel with f16
+    (1537, 256, 2048, binding.EPI_BIAS_RELU_F16),     # long K with f16 operands
     (333, 1024, 136, binding.EPI_BIAS_RESID_RELU_F16),
     (6272, 2048, 512, binding.EPI_BIAS_RESID_RELU_F16),  # last conv3 of ResNet-50 at batch 128
 ]
